@@ -77,9 +77,10 @@ __device__ inline float warp_min_f(float v) {
 }
 
 // Must be called by all 32 lanes of the warp with the same query.  `t` is each lane's own
-// nearest state (test1 / range over triangle indices; r2(): its squared radius rounded up to
-// float); `box(lx, ly, lz, hx, hy, hz)` returns a lower bound of the squared distance from the
-// query point to a box, rounded down to float.  s_code / s_e: this warp's kCoopStack entries
+// nearest state (coop_range over triangle indices; coop_r2(): its squared radius rounded up to
+// float); `box(lx, ly, lz, hx, hy, hz, r2)` returns a lower bound of the squared distance from
+// the query point to a box, rounded down to float (r2, the warp's squared radius, lets it
+// stop at a coarser bound that decides the comparison).  s_code / s_e: this warp's kCoopStack entries
 // (node index, box bound).  With kCut, the traversal stops early, returning true, once the
 // warp's squared radius is below cut2 (cut_radius).  The two forms are separate
 // instantiations, chosen per query: the loop without the checks is compiled as if they did
@@ -133,7 +134,7 @@ __device__ inline bool traverse_coop(const BvhDev& B, Near& t, const Box& box, u
       if (code != kNoChild) {
         ++c.boxes;
         e = box(__ldg(nf + ch), __ldg(nf + 4 + ch), __ldg(nf + 8 + ch), __ldg(nf + 12 + ch), __ldg(nf + 16 + ch),
-                __ldg(nf + 20 + ch));
+                __ldg(nf + 20 + ch), r2);
       }
     }
     const bool hit = code != kNoChild && e <= r2;
@@ -145,7 +146,7 @@ __device__ inline bool traverse_coop(const BvhDev& B, Near& t, const Box& box, u
       lq += __popc(lm);
     }
 #else
-    if (hit && code_count(code) > 0) t.range(code_ref(code), code_count(code));
+    if (hit && code_count(code) > 0) t.coop_range(code_ref(code), code_count(code), r2);
     r2 = warp_min_f(t.coop_r2());
     if constexpr (kCut) {
       if (r2 < cut2) return true;
@@ -206,7 +207,7 @@ __device__ inline bool traverse_coop(const BvhDev& B, Near& t, const Box& box, u
       const int take = min(lq, 32);
       if (lane < take) {
         const unsigned code = lq_code[lq - take + lane];
-        t.range(code_ref(code), code_count(code));
+        t.coop_range(code_ref(code), code_count(code), r2);
       }
       lq -= take;
       __syncwarp();  // the entries taken are read before new ones overwrite them

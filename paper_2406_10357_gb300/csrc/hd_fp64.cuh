@@ -2,115 +2,32 @@
 // arithmetic of the paper's implementation (Section 4).
 #pragma once
 
+#include "hd_cert.cuh"
 #include "hd_coop.cuh"
 #include "hd_internal.cuh"
 
 namespace hd {
 
-constexpr int kStack = 96;  // up to 3 pushes per 4-wide node
+constexpr int kStack = 96;  // up to 4 pushes per 4-wide node, one of them popped next
 
-// Nearest triangle of B to p by ordered depth-first traversal of the BVH: both child
-// boxes come with one node fetch, leaf children are tested at once, the nearer internal
-// child is entered and the farther one pushed with its box distance, which is re-checked
-// when popped.  `Test` gets a triangle range and may shrink the pruning radius it holds.
-// Returns kTravOver once `test` has tested more than `budget` triangles, and kTravCut once
-// its squared radius is below test.cut2 (cut_radius), with the traversal unfinished (what
-// `test` holds is then the best triangle found so far); kTravDone when it finished.
-constexpr int kTravDone = 0, kTravOver = 1, kTravCut = 2;
-template <bool kCut, class Test>
-__device__ inline int traverse(const BvhDev& B, D3 p, Test& test, Counters& c, int budget = INT_MAX) {
-  int stack_node[kStack];
-  double stack_d[kStack];
-  int sp = 0;
-  int node = 0;
-  for (;;) {
-    if ((int)test.evals > budget) return kTravOver;
-    if constexpr (kCut) {
-      if (test.radius2() < test.cut2) return kTravCut;
-    }
-    const float4* np = reinterpret_cast<const float4*>(B.nodes + node);
-    const float4 lx = __ldg(np), ly = __ldg(np + 1), lz = __ldg(np + 2);
-    const float4 hx = __ldg(np + 3), hy = __ldg(np + 4), hz = __ldg(np + 5);
-    const uint4 cd = __ldg(reinterpret_cast<const uint4*>(np + 6));
-    ++c.nodes;
-    double e[4] = {box_dist2(p, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x), box_dist2(p, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y),
-                   box_dist2(p, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z), box_dist2(p, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w)};
-    unsigned k[4] = {cd.x, cd.y, cd.z, cd.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      c.boxes += k[j] != kNoChild;
-      if (k[j] == kNoChild) e[j] = INFINITY;
-    }
-    // nearest first (sorting network on four)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int a = q == 0 ? 0 : q == 1 ? 2 : q == 2 ? 0 : q == 3 ? 1 : 1;
-      const int b = q == 0 ? 1 : q == 1 ? 3 : q == 2 ? 2 : q == 3 ? 3 : 2;
-      if (e[b] < e[a]) {
-        double te = e[a];
-        e[a] = e[b];
-        e[b] = te;
-        unsigned tk = k[a];
-        k[a] = k[b];
-        k[b] = tk;
-      }
-    }
-    if constexpr (kCut) {
-      // a child box wholly within the cut radius: one of its triangles is close enough
-      const uint4 rp = __ldg(reinterpret_cast<const uint4*>(np + 7));
-      const float px = (float)p.x, py = (float)p.y, pz = (float)p.z;
-      const float c2 = (float)test.cut2;
-      int pick = -1;
-      if (cd.w != kNoChild && box_far2(px, py, pz, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w) < c2) pick = (int)rp.w;
-      if (cd.z != kNoChild && box_far2(px, py, pz, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z) < c2) pick = (int)rp.z;
-      if (cd.y != kNoChild && box_far2(px, py, pz, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y) < c2) pick = (int)rp.y;
-      if (cd.x != kNoChild && box_far2(px, py, pz, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x) < c2) pick = (int)rp.x;
-      if (pick >= 0) {
-        test.range(pick, 1);
-        if (test.radius2() < test.cut2) return kTravCut;
-      }
-    }
-    // leaf ranges first, nearest first, so that the radius shrinks before the inner
-    // children are kept or dropped
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (k[j] != kNoChild && code_count(k[j]) > 0 && e[j] < test.radius2()) test.range(code_ref(k[j]), code_count(k[j]));
-    const double r2 = test.radius2();
-    int next = -1;
-    double next_d = 0.0;
-#pragma unroll
-    for (int j = 3; j >= 0; --j) {  // farthest inner children pushed first; the nearest is taken
-      if (k[j] == kNoChild || code_count(k[j]) > 0 || !(e[j] < r2)) continue;
-      if (next >= 0) {
-        if (sp < kStack) {
-          stack_node[sp] = next;
-          stack_d[sp] = next_d;
-          ++sp;
-        } else {
-          c.err = 1;  // stack overflow: the subtree is skipped and the error reported
-        }
-      }
-      next = code_ref(k[j]);
-      next_d = e[j];
-    }
-    if (next >= 0) {
-      node = next;
-      continue;
-    }
-    bool found = false;
-    while (sp > 0) {
-      --sp;
-      if (stack_d[sp] < test.radius2()) {
-        node = stack_node[sp];
-        found = true;
-        break;
-      }
-    }
-    if (!found) break;
-  }
-  return kTravDone;
+// Squared distance from p to triangle j of B, with the closest point, in FP64.
+static __device__ __forceinline__ double tri_dist2(const double* tri64, const float4* tri32, int j, D3 p, D3& x) {
+  D3 a, b, c;
+  load_tri_d(tri64, tri32, j, a, b, c);
+  x = closest_on_triangle(p, a, b, c);
+  const D3 e = p - x;
+  return dot(e, e);
 }
 
+
+// The nearest-triangle state of one query in FP64, with FP32 filters.  FP64 arithmetic runs
+// at 1/64 of the FP32 rate on GB300, so the traversal decides everything it can from
+// certified FP32 intervals (box distances, and a lower bound of each leaf triangle's
+// distance) and takes an FP64 step only where the interval leaves the decision open: the
+// point-triangle test of a triangle that may be nearer than the best so far, and the box
+// distance where it is within FP32 rounding of the radius or of another child's.  Every
+// decision is thus the one the same traversal in FP64 alone takes, so the triangles tested,
+// the order among equal distances, the budget and the result are bit for bit its own.
 struct NearestD {
   D3 p;
   const double* tri64;
@@ -119,26 +36,288 @@ struct NearestD {
   double cut2 = -1.0;  // the traversal may stop once best2 < cut2 (cut_radius)
   int best = -1;
   D3 q = {0, 0, 0};
-  unsigned evals = 0;
-  __device__ double radius2() const { return best2; }
-  __device__ float coop_r2() const { return __double2float_ru(best2); }
+  unsigned evals = 0;  // triangles tested (by the filter, and in FP64 where it leaves them open)
+  FFP P;               // p as a float pair
+  float guard = 0.f;   // what the float forms of p and B and the FP64 test's own rounding can hide
+  float pmax = 0.f;
+  // best2 rounded down / up to float, and its square root rounded up
+  float r2lo = INFINITY, r2hi = INFINITY, rhi = INFINITY;
+
+  __device__ void start(const BvhDev& B, double x, double y, double z) {
+    p = {x, y, z};
+    tri64 = B.tri64;
+    tri32 = B.tri32;
+    P.h = {__double2float_rn(x), __double2float_rn(y), __double2float_rn(z)};
+    P.l = {__double2float_rn(x - (double)P.h.x), __double2float_rn(y - (double)P.h.y),
+           __double2float_rn(z - (double)P.h.z)};
+    // |p - (h + l)| <= 2^-48 |p| (1e-37 where l underflows), the FP64 test rounds within
+    // 2^-48 of the coordinates it works on, and B's float vertices lie within eta of its own
+    guard = __fadd_ru(__ldg(B.meta), 1e-37f);
+    pmax = amax3(P.h);
+  }
+  // Enclosure of p on each axis, for the box intervals.
+  __device__ F3 below() const {
+    return {__double2float_rd(p.x), __double2float_rd(p.y), __double2float_rd(p.z)};
+  }
+  __device__ F3 above() const {
+    return {__double2float_ru(p.x), __double2float_ru(p.y), __double2float_ru(p.z)};
+  }
+  __device__ void set_radius() {
+    r2lo = __double2float_rd(best2);
+    r2hi = __double2float_ru(best2);
+    rhi = sqrt_up(r2hi);
+  }
+  __device__ float coop_r2() const { return r2hi; }
+  // Whether triangle j may be nearer than r (false: its FP64 squared distance is certainly
+  // not below r^2).
+  __device__ bool may(int j, float r) const {
+    const float4* t = tri32 + 3 * (size_t)j;
+    float M;
+    const float lo = pt_lo(P, __ldg(t), __ldg(t + 1), __ldg(t + 2), M);
+    return !(__fsub_rd(lo, __fmaf_ru(0x1p-40f, __fadd_ru(pmax, M), guard)) > r);
+  }
   __device__ void test1(int j) {
-    D3 a, b, c;
-    load_tri_d(tri64, tri32, j, a, b, c);
-    D3 x = closest_on_triangle(p, a, b, c);
-    D3 e = p - x;
-    double d2 = dot(e, e);
-    ++evals;
+    D3 x;
+    const double d2 = tri_dist2(tri64, tri32, j, p, x);
     if (d2 < best2) {
       best2 = d2;
       best = j;
       q = x;
+      set_radius();
     }
   }
-  __device__ void range(int first, int count) {
-    for (int j = first; j < first + count; ++j) test1(j);
+  // A leaf range in the cooperative traversal; r2 is the warp's squared radius.
+  __device__ void coop_range(int first, int count, float r2) {
+    const float r = sqrt_up(r2);
+    for (int j = first; j < first + count; ++j) {
+      ++evals;
+      if (may(j, fminf(r, rhi))) test1(j);
+    }
   }
 };
+
+// Nearest triangle of B to t.p by ordered depth-first traversal of the BVH: a node's leaf
+// children are tested first, nearest first, then its inner children are entered nearest
+// first, each while its box lies within the radius of the moment.  Must be called by all 32
+// lanes of the warp; inactive lanes start finished.  `first` (or -1) is a triangle to test
+// before the traversal.
+//
+// The lanes go in three steps, so that each kind of work runs on as many of them as
+// possible: a lane expands nodes until it has a leaf triangle pending; the lanes that have
+// one filter it in FP32; a lane whose triangle passes waits, and once every lane waits or is
+// finished they run the FP64 test together.  (Tested at once, the few triangles of each lane
+// that need FP64 would each cost the whole warp a test of its own.)
+//
+// Bound by the FP64 pipe (2 lanes per clock and SM) before the filters: every node cost four
+// FP64 box distances, every leaf triangle an FP64 test.  Round 0 and one round of the torus
+// pair (200,000 vs 50,176 triangles, 203,860 queries): 2.20 -> 0.72 ms; 40,001 points through
+// the torus's volume (two thirds finished by warps): 3.49 -> 1.24 ms.
+//
+// Returns kTravOver once more than `budget` triangles have been tested, and kTravCut once the
+// squared radius is below t.cut2 (cut_radius), with the traversal unfinished (t then holds
+// the best triangle found so far); kTravDone when it finished.
+constexpr int kTravDone = 0, kTravOver = 1, kTravCut = 2;
+template <bool kCut>
+__device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool active, int first, int budget) {
+  unsigned stack_node[kStack];
+  float2 stack_e[kStack];  // the interval of each entry's squared box distance
+  int sp = 0;
+  int node = active ? 0 : -1;  // inner node to expand next
+  int leaf_node = 0, slots = 0, n_slots = 0;  // leaf children waiting: their slots in leaf_node, 2 bits each
+  int lfirst = 0, lcount = 0;                 // leaf triangles waiting
+  bool picked = false;                        // kCut: the waiting triangle is a cut query's pick
+  int need = active ? first : -1;             // triangle waiting for its FP64 test
+  if (need >= 0) ++t.evals;
+  bool done = !active;
+  int how = kTravDone;
+  const F3 plo = t.below(), phi = t.above();
+  for (;;) {
+    while (!done && need < 0 && n_slots == 0 && lcount == 0 && !picked) {
+      bool open = false;  // node's own box distance is within rounding of the radius
+      if (node < 0) {
+        while (sp > 0) {
+          --sp;
+          const float2 e = stack_e[sp];
+          if (e.x > t.r2hi) continue;
+          node = (int)stack_node[sp];
+          open = !(e.y < t.r2lo);
+          break;
+        }
+        if (node < 0) {
+          done = true;
+          continue;
+        }
+      }
+      const float4* np = reinterpret_cast<const float4*>(B.nodes + node);
+      const float4 lx = __ldg(np), ly = __ldg(np + 1), lz = __ldg(np + 2);
+      const float4 hx = __ldg(np + 3), hy = __ldg(np + 4), hz = __ldg(np + 5);
+      const uint4 cd = __ldg(reinterpret_cast<const uint4*>(np + 6));
+      if (open) {  // its box is the union of its children's
+        const double e = box_dist2(t.p, fminf(fminf(lx.x, lx.y), fminf(lx.z, lx.w)),
+                                   fminf(fminf(ly.x, ly.y), fminf(ly.z, ly.w)),
+                                   fminf(fminf(lz.x, lz.y), fminf(lz.z, lz.w)),
+                                   fmaxf(fmaxf(hx.x, hx.y), fmaxf(hx.z, hx.w)),
+                                   fmaxf(fmaxf(hy.x, hy.y), fmaxf(hy.z, hy.w)),
+                                   fmaxf(fmaxf(hz.x, hz.y), fmaxf(hz.z, hz.w)));
+        if (!(e < t.best2)) {
+          node = -1;
+          continue;
+        }
+      }
+      if ((int)t.evals > budget) {
+        how = kTravOver;
+        done = true;
+        continue;
+      }
+      if constexpr (kCut) {
+        if (t.best2 < t.cut2) {
+          how = kTravCut;
+          done = true;
+          continue;
+        }
+      }
+      ++c.nodes;
+      // the children's intervals; those certainly beyond the radius, and missing ones, at +inf
+      float el[4], eh[4];
+      int sl[4] = {0, 1, 2, 3};
+      auto child = [&](int j, unsigned k, float ax, float ay, float az, float bx, float by, float bz) {
+        el[j] = box_lo2(plo, phi, ax, ay, az, bx, by, bz);
+        eh[j] = box_hi2(plo, phi, ax, ay, az, bx, by, bz);
+        c.boxes += k != kNoChild;
+        if (k == kNoChild || el[j] > t.r2hi) el[j] = eh[j] = INFINITY;
+      };
+      child(0, cd.x, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x);
+      child(1, cd.y, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y);
+      child(2, cd.z, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z);
+      child(3, cd.w, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w);
+      // nearest first (sorting network on four: a pair is swapped when the later child is nearer)
+      bool tie = false;  // an order the intervals leave open
+#pragma unroll
+      for (int s = 0; s < 5; ++s) {
+        const int a = s == 0 ? 0 : s == 1 ? 2 : s == 2 ? 0 : s == 3 ? 1 : 1;
+        const int b = s == 0 ? 1 : s == 1 ? 3 : s == 2 ? 2 : s == 3 ? 3 : 2;
+        if (eh[b] < el[a]) {
+          const float x = el[a], y = eh[a];
+          el[a] = el[b];
+          eh[a] = eh[b];
+          el[b] = x;
+          eh[b] = y;
+          const int k = sl[a];
+          sl[a] = sl[b];
+          sl[b] = k;
+        } else {
+          tie |= el[b] <= eh[a] && eh[a] > 0.f && el[a] < INFINITY && el[b] < INFINITY;
+        }
+      }
+      if (tie) {  // rare: the same network on the FP64 distances
+        double e[4];
+        auto exact = [&](int j, unsigned k, float ax, float ay, float az, float bx, float by, float bz) {
+          e[j] = k == kNoChild ? INFINITY : box_dist2(t.p, ax, ay, az, bx, by, bz);
+          sl[j] = j;
+        };
+        exact(0, cd.x, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x);
+        exact(1, cd.y, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y);
+        exact(2, cd.z, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z);
+        exact(3, cd.w, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w);
+#pragma unroll
+        for (int s = 0; s < 5; ++s) {
+          const int a = s == 0 ? 0 : s == 1 ? 2 : s == 2 ? 0 : s == 3 ? 1 : 1;
+          const int b = s == 0 ? 1 : s == 1 ? 3 : s == 2 ? 2 : s == 3 ? 3 : 2;
+          if (e[b] < e[a]) {
+            const double x = e[a];
+            e[a] = e[b];
+            e[b] = x;
+            const int k = sl[a];
+            sl[a] = sl[b];
+            sl[b] = k;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          el[j] = __double2float_rd(e[j]);
+          eh[j] = __double2float_ru(e[j]);
+          if (el[j] > t.r2hi) el[j] = eh[j] = INFINITY;
+        }
+      }
+      if constexpr (kCut) {
+        // a child box wholly within the cut radius: one of its triangles is close enough
+        const uint4 rp = __ldg(reinterpret_cast<const uint4*>(np + 7));
+        const float px = t.P.h.x, py = t.P.h.y, pz = t.P.h.z;
+        const float c2 = (float)t.cut2;
+        int pick = -1;
+        if (cd.w != kNoChild && box_far2(px, py, pz, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w) < c2) pick = (int)rp.w;
+        if (cd.z != kNoChild && box_far2(px, py, pz, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z) < c2) pick = (int)rp.z;
+        if (cd.y != kNoChild && box_far2(px, py, pz, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y) < c2) pick = (int)rp.y;
+        if (cd.x != kNoChild && box_far2(px, py, pz, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x) < c2) pick = (int)rp.x;
+        if (pick >= 0) {
+          lfirst = pick;
+          lcount = 1;
+          picked = true;
+        }
+      }
+      // the inner children go on the stack, farthest first; the leaves wait, nearest first
+      // (their tests come first and shrink the radius the stack is popped with)
+      leaf_node = node;
+      slots = 0;
+#pragma unroll
+      for (int j = 3; j >= 0; --j) {
+        if (!(el[j] < INFINITY)) continue;
+        const unsigned k = sl[j] == 0 ? cd.x : sl[j] == 1 ? cd.y : sl[j] == 2 ? cd.z : cd.w;
+        if (code_count(k) > 0) {
+          slots = (slots << 2) | sl[j];
+          ++n_slots;
+        } else if (sp < kStack) {
+          stack_node[sp] = (unsigned)code_ref(k);
+          stack_e[sp] = make_float2(el[j], eh[j]);
+          ++sp;
+        } else {
+          c.err = 1;  // stack overflow: the subtree is skipped and the error reported
+        }
+      }
+      node = -1;
+    }
+    if (!done && need < 0) {
+      if (lcount == 0) {
+        if (kCut && picked) {
+          picked = false;
+          if (t.best2 < t.cut2) {
+            how = kTravCut;
+            done = true;
+          }
+        }
+        if (!done && n_slots > 0) {
+          const int s = slots & 3;
+          slots >>= 2;
+          --n_slots;
+          const float* nf = reinterpret_cast<const float*>(B.nodes + leaf_node) + s;
+          const float ax = __ldg(nf), ay = __ldg(nf + 4), az = __ldg(nf + 8);
+          const float bx = __ldg(nf + 12), by = __ldg(nf + 16), bz = __ldg(nf + 20);
+          const unsigned k = __ldg(reinterpret_cast<const unsigned*>(nf) + 24);
+          bool in = box_hi2(plo, phi, ax, ay, az, bx, by, bz) < t.r2lo;
+          if (!in && !(box_lo2(plo, phi, ax, ay, az, bx, by, bz) > t.r2hi))
+            in = box_dist2(t.p, ax, ay, az, bx, by, bz) < t.best2;
+          if (in) {
+            lfirst = code_ref(k);
+            lcount = code_count(k);
+          }
+        }
+      }
+      if (!done && lcount > 0) {
+        ++t.evals;
+        if (t.may(lfirst, t.rhi)) need = lfirst;
+        ++lfirst;
+        --lcount;
+      }
+    }
+    if (__any_sync(0xffffffffu, !done && need < 0)) continue;
+    if (__all_sync(0xffffffffu, done)) break;
+    if (need >= 0) {
+      t.test1(need);
+      need = -1;
+    }
+  }
+  return how;
+}
 
 __device__ inline double dist_to_tri64(const BvhDev& B, int j, D3 x) {
   D3 a, b, c;
@@ -181,37 +360,6 @@ __device__ inline double ub_u2(const VI t[3]) {
     if (s - r > 2.0 * R) g = R;
   }
   return g + fmax(t[0].d, fmax(t[1].d, t[2].d));
-}
-
-// Shared edge of triangles f, g of B (equal vertex indices of their F_B rows): returns
-// true with the slots of the two shared vertices in f and the opposite slots in f and g.
-__device__ inline bool shared_edge(const BvhDev& B, int f, int g, int& fs0, int& fs1, int& fo, int& go) {
-  int4 a = __ldg(B.tri_vid + f), b = __ldg(B.tri_vid + g);
-  int av[3] = {a.x, a.y, a.z}, bv[3] = {b.x, b.y, b.z};
-  bool ash[3];
-  int nsh = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) ash[i] = (av[i] == bv[0] || av[i] == bv[1] || av[i] == bv[2]);
-  // distinct shared vertex indices of f
-  int sl[3], ns = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (!ash[i]) continue;
-    bool dup = false;
-    for (int k = 0; k < ns; ++k) dup |= av[sl[k]] == av[i];
-    if (!dup) sl[ns++] = i;
-  }
-  nsh = ns;
-  if (nsh != 2) return false;
-  fs0 = sl[0];
-  fs1 = sl[1];
-  fo = go = -1;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (av[i] != av[fs0] && av[i] != av[fs1]) fo = i;
-    if (bv[i] != av[fs0] && bv[i] != av[fs1]) go = i;
-  }
-  return fo >= 0 && go >= 0;
 }
 
 __device__ inline D3 tri_vertex(const BvhDev& B, int j, int slot) {
@@ -365,24 +513,29 @@ struct PolicyD {
   static constexpr int kLongBudget = HD_LONG_BUDGET_D;      // triangle tests of a lane before the hand-off
   static constexpr int kBoundRegs = HD_FP64_BOUND_REGS;  // register cap of the UpperBound kernels
 
-  // Nearest triangle of v.  With `over` given, a traversal that tests more than `budget`
-  // triangles stops, sets *over and leaves its best triangle so far in v (hint, d = its
-  // squared distance, q) for query_coop to finish.
+  // Nearest triangle of v.  Called by every lane of the warp (the traversal votes over the
+  // full warp); lanes with active == false only vote and leave v untouched.  With `over`
+  // given, a traversal that tests more than `budget` triangles stops, sets *over and leaves
+  // its best triangle so far in v (hint, d = its squared distance, q) for query_coop to finish.
   // With cut_r >= 0 (cut_radius), the query may stop at a triangle within cut_r of v: it
   // then sets *was_cut and keeps that triangle and its distance (not a lower bound then).
   __device__ static void query(const BvhDev& B, Vtx& v, Counters& c, bool active, int budget = INT_MAX,
                                bool* over = nullptr, double cut_r = -1.0, bool* was_cut = nullptr) {
-    if (!active) return;  // no warp-collective operations below
     NearestD t;
-    t.p = {v.x, v.y, v.z};
-    t.tri64 = B.tri64;
-    t.tri32 = B.tri32;
-    if (cut_r > 0.0) t.cut2 = cut_r * cut_r;
-    // start from the hint, or from a triangle of the point's grid cell (a first radius)
-    const int h0 = v.hint >= 0 ? v.hint : grid_hint(B, (float)v.x, (float)v.y, (float)v.z);
-    if (h0 >= 0) t.test1(h0);
-    if (v.hint < 0 && h0 >= 0 && budget < INT_MAX) ++budget;  // the grid's triangle is not the traversal's
-    const int how = cut_r > 0.0 ? traverse<true>(B, t.p, t, c, budget) : traverse<false>(B, t.p, t, c, budget);
+    int h0 = -1;
+    if (active) {
+      t.start(B, v.x, v.y, v.z);
+      if (cut_r > 0.0) t.cut2 = cut_r * cut_r;
+      // start from the hint, or from a triangle of the point's grid cell (a first radius)
+      h0 = v.hint >= 0 ? v.hint : grid_hint(B, t.P.h.x, t.P.h.y, t.P.h.z);
+      if (v.hint < 0 && h0 >= 0 && budget < INT_MAX) ++budget;  // the grid's triangle is not the traversal's
+    } else {
+      t.p = {0.0, 0.0, 0.0};
+    }
+    // one instantiation for the whole warp
+    const int how = __any_sync(0xffffffffu, t.cut2 > 0.0) ? traverse<true>(B, t, c, active, h0, budget)
+                                                          : traverse<false>(B, t, c, active, h0, budget);
+    if (!active) return;
     c.leaf += t.evals;
     if (how == kTravCut && was_cut) *was_cut = true;
     if (how == kTravOver) {
@@ -408,16 +561,20 @@ struct PolicyD {
                                     double cut_r = -1.0) {
     const int lane = threadIdx.x & 31;
     NearestD t;
-    t.p = {v.x, v.y, v.z};
-    t.tri64 = B.tri64;
-    t.tri32 = B.tri32;
+    t.start(B, v.x, v.y, v.z);
     if (lane == 0 && v.hint >= 0) {  // the lane traversal's best so far
       t.best = v.hint;
       t.best2 = v.d;
       t.q = {v.qx, v.qy, v.qz};
+      t.set_radius();
     }
+    // the FP64 squared box distance rounded down to float decides (e <= r2); where its FP32
+    // interval lies on one side of r2, the interval's lower end decides the same
     const D3 p = t.p;
-    auto box = [p](float lx, float ly, float lz, float hx, float hy, float hz) {
+    const F3 plo = t.below(), phi = t.above();
+    auto box = [p, plo, phi](float lx, float ly, float lz, float hx, float hy, float hz, float r2) {
+      const float e = box_lo2(plo, phi, lx, ly, lz, hx, hy, hz);
+      if (e > __fmul_ru(r2, 1.f + 4.f * kU) || box_hi2(plo, phi, lx, ly, lz, hx, hy, hz) <= r2) return e;
       return __double2float_rd(box_dist2(p, lx, ly, lz, hx, hy, hz));
     };
     const float cut2 = cut_r > 0.0 ? __double2float_rd(cut_r * cut_r) : 0.f;
