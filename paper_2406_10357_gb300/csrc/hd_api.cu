@@ -166,7 +166,12 @@ __global__ void k_upper_bounds(BvhDev B, const int* inv, const double* T, const 
   }
   unsigned ev = 0;
   int c;
-  U[i] = upper_bound_d(B, t, l, rp.order, rp.n_bounds, c, ev);
+  double own[3];  // the distances given need not be those to the triangles given
+  for (int k = 0; k < 3; ++k) {
+    D3 x;
+    own[k] = sqrt(tri_dist2(B.tri64, B.tri32, t[k].I, t[k].v, x));
+  }
+  U[i] = upper_bound_d(B, t, own, l, rp.order, rp.n_bounds, true, c, ev);
   code[i] = c;
 }
 

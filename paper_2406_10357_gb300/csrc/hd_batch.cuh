@@ -47,7 +47,7 @@ struct BatchState {
   int n_front;    // items in the current frontier (all pairs)
   int n_next;     // items appended to the next frontier
   int n_split;    // split slots taken this round
-  int n_u4;       // items in the u4 list (MIXED)
+  int n_u4;       // items left to the second pass of the bounds
   int n_promote;  // items handed to the FP64 phase (MIXED)
   int n_long;     // queries handed to the cooperative traversal by the last query launch
   int q_next, b_next, long_next;  // work counters of the query, bound and cooperative kernels
@@ -449,9 +449,10 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
         if (t < count) p = make(t, it, up);
         if (p >= 0) {
           const PairLevel<P> pl = pair_level<P>(x, p);
-          float U, u12;
+          typename P::UT U;
+          float u12;
           int code;
-          if (P::paper_cheap(pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.lv.lf, pl.rp, &U, &code, &u12)) {
+          if (P::paper_cheap(x.pd[p].B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.lv.lf, pl.rp, &U, &code, &u12)) {
             need = true;
             e = BatchRebinEntry{{it.v[0], it.v[1], it.v[2]}, u12, up, p};
           } else {
@@ -480,7 +481,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
         it.v[2] = e.v[2];
         const PairLevel<P> pl = pair_level<P>(x, p);
         int code;
-        const float U =
+        const typename P::UT U =
             P::paper_u3(x.pd[p].B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], pl.lv.lf, pl.rp, e.u12, code, cnt);
         it.U = e.up < U ? e.up : U;
         classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
@@ -567,7 +568,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
   }
 }
 
-// The u4 pass (MIXED): items whose cascade reached a trailing u4, with full warps.
+// The pass over the items the UpperBound kernel left (bound_u4_body), with full warps.
 template <class P>
 __global__ void k_batch_bound_u4(BatchCtx x, const typename P::Vtx* pool, const typename P::Item* u4list,
                                  const int* u4_pair, int cap, typename P::Item* next, int* next_pair, int next_cap,
@@ -582,21 +583,18 @@ __global__ void k_batch_bound_u4(BatchCtx x, const typename P::Vtx* pool, const 
        base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = base + (threadIdx.x & 31);
     int p = -1;
+    Counters cnt;
     PairTally<P> ty;
     if (t < n) {
       p = u4_pair[t];
       typename P::Item it = u4list[t];
       const PairLevel<P> pl = pair_level<P>(x, p);
-      const typename P::UT u = P::bound_u4(pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.rp, it.U);
-      int code = 5;
-      if (u < pl.lv.th.lo) {
-        code = 4;
-        it.U = u;
-      } else if (u < it.U) {
-        it.U = u;
-      }
+      int code;
+      P::bound_deferred(x.pd[p].B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.lv.l, pl.lv.th.lo, pl.rp, it.U, code,
+                        cnt);
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, nullptr, nullptr, ty);
     }
+    if constexpr (P::kFp64) flush_counters_pair(x.sts, p, cnt);
     flush_tally_pair<P>(x.sts, p, ty);
   }
 }
@@ -761,17 +759,15 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
   }
 }
 
-// The UpperBound kernels of policy P: the straight-line paper-order instantiation (MIXED only)
-// or the general one.
+// The UpperBound kernels of policy P: the straight-line paper-order instantiation or the
+// general one.
 template <class P>
 auto batch_faces_kernel(bool paper) {
-  if constexpr (P::kFp64) return k_batch_bound_faces<P, false>;
-  else return paper ? k_batch_bound_faces<P, true> : k_batch_bound_faces<P, false>;
+  return paper ? k_batch_bound_faces<P, true> : k_batch_bound_faces<P, false>;
 }
 template <class P>
 auto batch_children_kernel(bool paper) {
-  if constexpr (P::kFp64) return k_batch_bound_children<P, false>;
-  else return paper ? k_batch_bound_children<P, true> : k_batch_bound_children<P, false>;
+  return paper ? k_batch_bound_children<P, true> : k_batch_bound_children<P, false>;
 }
 
 // ----------------------------------------------------------------------------- round control
@@ -948,6 +944,9 @@ struct BatchBufs {
   int* split_pair = nullptr;
   typename P::Item* u4list = nullptr;  // MIXED only
   int* u4_pair = nullptr;
+  // the list of items left to the second pass of the bounds that fill front[to] (Rounds::left)
+  typename P::Item* left(int to) const { return u4list ? u4list : front[to ^ 1]; }
+  int* left_pair(int to) const { return u4list ? u4_pair : front_pair[to ^ 1]; }
   typename P::Item* promo = nullptr;   // MIXED only
   int* promo_pair = nullptr;
   LongList longq = {nullptr, 0};
@@ -1048,7 +1047,7 @@ int batch_rounds(const BatchCtx& x, BatchBufs<P>& R, const BatchCtl& c, int n_po
     const int rh = batch_host_res(hr);
     if (rh != HD_OK) return rh;
   }
-  const bool paper = !P::kFp64 && paper_cascade(x.rp);
+  const bool paper = paper_cascade(x.rp);
   auto k_children = batch_children_kernel<P>(paper);
   const size_t smem_b = batch_rebin_smem(bs_);  // the u3 queues of the paper-order kernels
   const unsigned g_q = batch_grid(k_batch_query<P>, bs_, sms), g_b = batch_grid(k_children, bs_, sms, smem_b);
@@ -1076,10 +1075,10 @@ int batch_rounds(const BatchCtx& x, BatchBufs<P>& R, const BatchCtl& c, int n_po
     {
       TraceScope tr(HD_K_BOUND, s);
       launch_chained(k_children, g_b, bs_, smem_b, s, x, R.pool, R.split_par, (const int*)R.split_pair, R.front[cur ^ 1],
-                     R.front_pair[cur ^ 1], (int)R.front_cap, R.u4list, R.u4_pair);
-      if (R.u4list)
-        launch_chained(k_batch_bound_u4<P>, g_u4, bs_, 0, s, x, R.pool, R.u4list, (const int*)R.u4_pair, (int)R.front_cap,
-                       R.front[cur ^ 1], R.front_pair[cur ^ 1], (int)R.front_cap, true);
+                     R.front_pair[cur ^ 1], (int)R.front_cap, R.left(cur ^ 1), R.left_pair(cur ^ 1));
+      launch_chained(k_batch_bound_u4<P>, g_u4, pass_block<P>(bs_), 0, s, x, R.pool,
+                     (const typename P::Item*)R.left(cur ^ 1), (const int*)R.left_pair(cur ^ 1), (int)R.front_cap,
+                     R.front[cur ^ 1], R.front_pair[cur ^ 1], (int)R.front_cap, true);
     }
     HD_TRY_LAUNCH();
     cur ^= 1;
@@ -1128,7 +1127,6 @@ int batch_finish_fp64(const BatchCtx& xm, BatchBufs<P>& RM, int64_t n_pro, const
   BatchCtx x = xm;
   x.nV = (int)(3 * n_pro);
   x.nF = (int)n_pro;
-  x.rp.defer_u4 = 0;
   auto fail = [&](cudaError_t err, const char* what) {
     cudaFreeAsync(tris, s);
     cudaFreeAsync(D.base, s);
@@ -1156,9 +1154,12 @@ int batch_finish_fp64(const BatchCtx& xm, BatchBufs<P>& RM, int64_t n_pro, const
   }
   {
     TraceScope tr(HD_K_BOUND, s);
-    launch_chained(k_batch_bound_faces<PolicyD, false>, blocks_for(n_pro, bsz), bsz, 0, s, x,
-                   (const VtxD*)D.pool, (const int32_t*)tris, (const int*)tri_pair, (int)n_pro, D.front[1],
-                   D.front_pair[1], (int)D.front_cap, (ItemD*)nullptr, (int*)nullptr);
+    launch_chained(batch_faces_kernel<PolicyD>(paper_cascade(x.rp)), blocks_for(n_pro, bsz), bsz, batch_rebin_smem(bsz),
+                   s, x, (const VtxD*)D.pool, (const int32_t*)tris, (const int*)tri_pair, (int)n_pro, D.front[1],
+                   D.front_pair[1], (int)D.front_cap, D.left(1), D.left_pair(1));
+    launch_chained(k_batch_bound_u4<PolicyD>, (unsigned)sms * 8, pass_block<PolicyD>(bsz), 0, s, x, (const VtxD*)D.pool,
+                   (const ItemD*)D.left(1), (const int*)D.left_pair(1), (int)D.front_cap, D.front[1], D.front_pair[1],
+                   (int)D.front_cap, false);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(e, "launch");
@@ -1270,7 +1271,7 @@ int run_batch(const hd_bvh* const* Bs, const hd_mesh* As, int64_t npairs, double
   rp.slack = 0.0;
   rp.slack_f = 0.f;
   rp.dyn = nullptr;
-  rp.defer_u4 = P::kFp64 ? 0 : 1;
+  rp.defer_u4 = 1;
   rp.parent_clamp = (o.flags & HD_FLAG_NO_PARENT_CLAMP) ? 0 : 1;
   memcpy(rp.order, o.order, 4);
   rp.n_bounds = o.n_bounds;
@@ -1290,7 +1291,7 @@ int run_batch(const hd_bvh* const* Bs, const hd_mesh* As, int64_t npairs, double
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int bsz = o.block_size;
-  const bool paper = !P::kFp64 && paper_cascade(rp);
+  const bool paper = paper_cascade(rp);
   // round 0 of every pair: validation, boxes, pool entries, eps; vertex queries; face bounds
   {
     TraceScope tr(HD_K_PREP, s);
@@ -1316,11 +1317,10 @@ int run_batch(const hd_bvh* const* Bs, const hd_mesh* As, int64_t npairs, double
     launch_chained(k_faces, std::min(blocks_for(nF, bsz), batch_grid(k_faces, bsz, sms, batch_rebin_smem(bsz))), bsz,
                    batch_rebin_smem(bsz), s, x,
                    (const typename P::Vtx*)R.pool, (const int32_t*)nullptr, (const int*)nullptr, 0, R.front[1],
-                   R.front_pair[1], (int)R.front_cap, R.u4list, R.u4_pair);
-    if (R.u4list)
-      launch_chained(k_batch_bound_u4<P>, (unsigned)sms * 8, bsz, 0, s, x, (const typename P::Vtx*)R.pool,
-                     (const typename P::Item*)R.u4list, (const int*)R.u4_pair, (int)R.front_cap, R.front[1],
-                     R.front_pair[1], (int)R.front_cap, false);
+                   R.front_pair[1], (int)R.front_cap, R.left(1), R.left_pair(1));
+    launch_chained(k_batch_bound_u4<P>, (unsigned)sms * 8, pass_block<P>(bsz), 0, s, x, (const typename P::Vtx*)R.pool,
+                   (const typename P::Item*)R.left(1), (const int*)R.left_pair(1), (int)R.front_cap, R.front[1],
+                   R.front_pair[1], (int)R.front_cap, false);
   }
   HD_TRY_LAUNCH();
   BatchCtl c;

@@ -686,7 +686,7 @@ __device__ inline Level<P> block_level(const RunState* st, double eps) {
 }
 
 // UpperBound of one sub-triangle: the cascade in the paper's order with u4 deferred
-// (kPaper, straight-line code, MIXED only), or in any order rp gives.
+// (kPaper, straight-line code), or in any order rp gives.
 template <class P, bool kPaper>
 __device__ inline typename P::UT bound_item(const BvhDev& B, const typename P::Vtx* pool, const typename P::Item& it,
                                             const Level<P>& lv, const RunParams& rp, int& code, Counters& c) {
@@ -744,9 +744,10 @@ __device__ inline void bound_rebin(const BvhDev& B, const typename P::Vtx* pool,
         typename P::Item it;
         float up = INFINITY;
         if (t < count && make(t, it, up)) {
-          float U, u12;
+          typename P::UT U;
+          float u12;
           int code;
-          if (P::paper_cheap(pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.lf, rp, &U, &code, &u12)) {
+          if (P::paper_cheap(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.lf, rp, &U, &code, &u12)) {
             need = true;
             e = RebinEntry{{it.v[0], it.v[1], it.v[2]}, u12, up};
           } else {
@@ -769,7 +770,7 @@ __device__ inline void bound_rebin(const BvhDev& B, const typename P::Vtx* pool,
         it.v[1] = e.v[1];
         it.v[2] = e.v[2];
         int code;
-        const float U = P::paper_u3(B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], lv.lf, rp, e.u12, code, c);
+        const typename P::UT U = P::paper_u3(B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], lv.lf, rp, e.u12, code, c);
         it.U = e.up < U ? e.up : U;
         classify<P>(st, it, lv.th, code, next, next_cap, u4list, ty);
       }
@@ -827,8 +828,9 @@ __global__ void HD_BOUND_REGS k_bound_faces(BvhDev B, const typename P::Vtx* poo
   flush_tally(st, ty);
 }
 
-// The u4 pass (MIXED): items whose cascade reached a trailing u4 get it here, in FP64, with
-// every lane of a warp on its own item; then discard / retire / keep as usual.
+// The pass over the items the UpperBound kernel left: those whose cascade reached a trailing
+// u4 (MIXED), or that the FP32 filter did not discard (FP64, the whole cascade), with every
+// lane of a warp on its own item; then discard / retire / keep as usual.
 template <class P>
 __device__ inline void bound_u4_body(BvhDev B, const typename P::Vtx* pool, const typename P::Item* u4list, int cap,
                            RunState* st, RunParams rp_in, typename P::Item* next, int next_cap) {
@@ -837,19 +839,15 @@ __device__ inline void bound_u4_body(BvhDev B, const typename P::Vtx* pool, cons
   int n = min(*(volatile int*)&st->n_u4, cap);
   const Level<P> lv = block_level<P>(st, rp.eps);
   const Thresholds<P>& th = lv.th;
+  Counters c;
   Tally<P> ty;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     typename P::Item it = u4list[t];
-    typename P::UT u = P::bound_u4(pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], rp, it.U);
-    int code = 5;
-    if (u < th.lo) {
-      code = 4;
-      it.U = u;
-    } else if (u < it.U) {
-      it.U = u;
-    }
+    int code;
+    P::bound_deferred(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.l, th.lo, rp, it.U, code, c);
     classify<P>(st, it, th, code, next, next_cap, nullptr, ty);
   }
+  if constexpr (P::kFp64) flush_counters(st, c);
   flush_tally(st, ty);
 }
 
@@ -1086,13 +1084,11 @@ inline bool paper_cascade(const RunParams& rp) {
 }
 template <class P>
 auto bound_faces_kernel(bool paper) {
-  if constexpr (P::kFp64) return k_bound_faces<P, false>;
-  else return paper ? k_bound_faces<P, true> : k_bound_faces<P, false>;
+  return paper ? k_bound_faces<P, true> : k_bound_faces<P, false>;
 }
 template <class P>
 auto bound_children_kernel(bool paper) {
-  if constexpr (P::kFp64) return k_bound_children<P, false>;
-  else return paper ? k_bound_children<P, true> : k_bound_children<P, false>;
+  return paper ? k_bound_children<P, true> : k_bound_children<P, false>;
 }
 
 // Per-loop constants of the round control.
@@ -1267,9 +1263,10 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_rounds(BvhDev B, TailBufs
     __syncthreads();
     query_long_body<P>(B, a.pool, lq, st, rp.slack, rp.dyn, true, s_code, s_e);
     __syncthreads();
-    bound_children_body<P>(B, a.pool, a.split_par, a.split_mid, st, rp, a.front[cur ^ 1], a.front_cap, a.u4list);
+    typename P::Item* left = a.u4list ? a.u4list : a.front[cur];
+    bound_children_body<P>(B, a.pool, a.split_par, a.split_mid, st, rp, a.front[cur ^ 1], a.front_cap, left);
     __syncthreads();
-    if (a.u4list) bound_u4_body<P>(B, a.pool, a.u4list, a.front_cap, st, rp, a.front[cur ^ 1], a.front_cap);
+    bound_u4_body<P>(B, a.pool, left, a.front_cap, st, rp, a.front[cur ^ 1], a.front_cap);
     __syncthreads();
     cur ^= 1;
     ++rounds;
@@ -1364,6 +1361,10 @@ struct Rounds {
   typename P::Item* front[2] = {nullptr, nullptr};
   typename P::Item* promo = nullptr;   // items handed to the FP64 phase (MIXED only)
   typename P::Item* u4list = nullptr;  // items waiting for the u4 pass (MIXED only)
+  // The list of items the UpperBound kernel leaves to its second pass while it fills
+  // front[to]: the u4 list, or (FP64) the other frontier buffer, which the round's select has
+  // read by then.
+  typename P::Item* left(int to) const { return u4list ? u4list : front[to ^ 1]; }
   int4* split_par = nullptr;
   int4* split_mid = nullptr;  // the three midpoint pool indices of every split
   MidTable tab = {nullptr, nullptr, nullptr, 0};
@@ -1372,6 +1373,13 @@ struct Rounds {
   int64_t n_pool = 0, n_front = 0;
   int cur = 1;  // front[cur] holds the current frontier
 };
+
+// Threads per block of the second pass of the bounds: the FP64 cascade's needs more registers
+// than the largest block sizes leave, and its FP64 pipe is kept busy by few warps.
+template <class P>
+constexpr int pass_block(int bs) {
+  return P::kFp64 ? 64 : bs;
+}
 
 // The largest block the round kernels of policy P launch with (their register use limits it
 // below 1024 threads).
@@ -1388,7 +1396,7 @@ int round_block_limit() {
       if (cudaFuncGetAttributes(&fa, bound_children_kernel<P>(paper)) == cudaSuccess)
         m = std::min(m, fa.maxThreadsPerBlock);
     }
-    if (cudaFuncGetAttributes(&fa, k_bound_u4<P>) == cudaSuccess) m = std::min(m, fa.maxThreadsPerBlock);
+    if (!P::kFp64 && cudaFuncGetAttributes(&fa, k_bound_u4<P>) == cudaSuccess) m = std::min(m, fa.maxThreadsPerBlock);
     m &= ~31;
     cached.store(m, std::memory_order_relaxed);
   }
@@ -1629,10 +1637,9 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     {
       TraceScope tr(HD_K_BOUND, s);
       launch_chained(k_children, g_b, bs, smem_b, s, B, R.pool, R.split_par, R.split_mid, st, rp, R.front[cur ^ 1],
-                     (int)R.front_cap, R.u4list);
-      if (R.u4list)
-        launch_chained(k_bound_u4<P>, g_u4, bs, 0, s, B, R.pool, R.u4list, (int)R.front_cap, st, rp, R.front[cur ^ 1],
-                                          (int)R.front_cap);
+                     (int)R.front_cap, R.left(cur ^ 1));
+      launch_chained(k_bound_u4<P>, g_u4, pass_block<P>(bs), 0, s, B, R.pool, (const typename P::Item*)R.left(cur ^ 1),
+                     (int)R.front_cap, st, rp, R.front[cur ^ 1], (int)R.front_cap);
     }
     HD_TRY_LAUNCH();
     cur ^= 1;
@@ -1741,6 +1748,7 @@ __global__ void k_promote_init(const typename P::Item* promo, int n, const typen
 static __global__ void k_phase_reset(RunState* st) {
   grid_dep_wait();
   grid_dep_launch();
+  st->stop = 0;  // the FP64 phase's own loop has not started
   st->q_next = 0;
   st->b_next = 0;
   st->n_next = 0;
@@ -1793,11 +1801,12 @@ int finish_in_fp64(const RunIO& io, Rounds<P>& RM, int64_t n_pro, RunState* st, 
   }
   {
     TraceScope tr(HD_K_BOUND, s);
-    RunParams rpd = rp;
-    rpd.defer_u4 = 0;
-    launch_chained(k_bound_faces<PolicyD>, blocks_for(n_pro, o.block_size), o.block_size, 0, s, B, D.pool, tris, n_pro, st, rpd,
-                                                                                   D.front[1], (int)D.front_cap,
-                                                                                   nullptr, 3 * n_pro);
+    const auto k_faces = bound_faces_kernel<PolicyD>(paper_cascade(rp));
+    launch_chained(k_faces, blocks_for(n_pro, o.block_size), o.block_size, rebin_smem(o.block_size), s, B, D.pool, tris,
+                   n_pro, st, rp, D.front[1], (int)D.front_cap, D.left(1), 3 * n_pro);
+    launch_chained(k_bound_u4<PolicyD>, blocks_for(n_pro, pass_block<PolicyD>(o.block_size)),
+                   pass_block<PolicyD>(o.block_size), 0, s, B, D.pool, (const ItemD*)D.left(1), (int)D.front_cap, st, rp,
+                   D.front[1], (int)D.front_cap);
   }
   HD_TRY_LAUNCH();
   D.cur = 1;
@@ -1860,7 +1869,7 @@ int run_bnb(const RunIO& io) {
   rp.slack = 0.0;
   rp.slack_f = 0.f;
   rp.dyn = dyn;
-  rp.defer_u4 = P::kFp64 ? 0 : 1;
+  rp.defer_u4 = 1;
   rp.parent_clamp = (o.flags & HD_FLAG_NO_PARENT_CLAMP) ? 0 : 1;
   memcpy(rp.order, o.order, 4);
   rp.n_bounds = o.n_bounds;
@@ -1889,10 +1898,9 @@ int run_bnb(const RunIO& io) {
     launch_chained(k_faces, std::min(blocks_for(io.nFA, bs), persistent_grid(k_faces, bs, sms, rebin_smem(bs))), bs,
                    rebin_smem(bs), s, 
         B, R.pool, io.FA, io.nFA, st, rp, R.front[1],
-                                                           (int)R.front_cap, R.u4list, io.nVA);
-    if (R.u4list)
-      launch_chained(k_bound_u4<P>, max_grid, bs, 0, s, B, R.pool, R.u4list, (int)R.front_cap, st, rp, R.front[1],
-                                            (int)R.front_cap);
+                                                           (int)R.front_cap, R.left(1), io.nVA);
+    launch_chained(k_bound_u4<P>, max_grid, pass_block<P>(bs), 0, s, B, R.pool, (const typename P::Item*)R.left(1),
+                   (int)R.front_cap, st, rp, R.front[1], (int)R.front_cap);
   }
   HD_TRY_LAUNCH();
 

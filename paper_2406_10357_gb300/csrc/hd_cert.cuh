@@ -18,6 +18,7 @@ __device__ inline F3 f3(float x, float y, float z) { return {x, y, z}; }
 __device__ inline F3 operator+(F3 a, F3 b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ inline F3 operator-(F3 a, F3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ inline float dotf(F3 a, F3 b) { return fmaf(a.x, b.x, fmaf(a.y, b.y, a.z * b.z)); }
+__device__ inline float sum1(F3 a) { return __fadd_ru(__fadd_ru(fabsf(a.x), fabsf(a.y)), fabsf(a.z)); }
 __device__ inline float amax3(F3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z))); }
 // Square root and quotient with outward rounding: the correctly rounded (round-to-nearest)
 // result is within half an ulp, so one multiplication by 1 +- 2^-23, rounded outward, bounds
@@ -337,6 +338,13 @@ __device__ inline FFP along(const VM& base, F3 e, float s, float& beta) {
 // point-triangle distances that are laid out as six evaluation slots, so that the lanes of a
 // warp run the same code whichever case each item is in: case 1 fills four slots, (b1, S1),
 // (b2, S1), (b1, S2), (b2, S2); case 2 fills all six with (v_j, S_i), j != i.
+//
+// With kAgree the value also bounds u3 with case 1's split points chosen in FP64 on B's own
+// coordinates: the points differ by at most the error of the split parameters times the edge,
+// which is added, and +inf is returned where rounding leaves open whether the split points or
+// the edge midpoints are used (a vertex of T close to the bisecting plane, as where A's edges
+// follow B's).
+template <bool kAgree = false>
 __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned& evals) {
   int lone = -1;
   if (!(t[0].I == t[1].I && t[1].I == t[2].I)) {
@@ -354,6 +362,7 @@ __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned
   const int S1 = v1.I, S2 = v2.I;
   FFP b1 = v1.p, b2 = v1.p;
   float be1 = 0.f, be2 = 0.f;
+  float apart = kAgree ? INFINITY : 0.f;  // kAgree: how far the FP64 split points may be from these
   if (c1) {
     F3 e12 = edge(v1, v2), e13 = edge(v1, v3);
     // split parameters: the bisecting plane of the two supporting half-planes (any value
@@ -378,6 +387,18 @@ __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned
         F3 nb = {w1.x * i1 - w2.x * i2, w1.y * i1 - w2.y * i2, w1.z * i1 - w2.z * i2};
         F3 r1 = (v1.p.h - p0) + v1.p.l;
         float sv1 = dotf(nb, r1), sv2 = sv1 + dotf(nb, e12), sv3 = sv1 + dotf(nb, e13);
+        if constexpr (kAgree) {
+          // the errors: of w1 and w2 relative to their lengths (the rounding of the projections,
+          // and eta in each vertex of B), hence of nb (|nb| <= 2), and of the side values
+          const float eta = __ldg(B.meta), n1 = sum1(a1), n2 = sum1(a2);
+          const float d = 2.f * ((32.f * kU * n1 + 4.f * eta * (1.f + n1 * ie)) * i1 +
+                                 (32.f * kU * n2 + 4.f * eta * (1.f + n2 * ie)) * i2) + 32.f * kU;
+          const float s1 = sum1(r1), s12 = sum1(e12), s13 = sum1(e13);
+          const float E1 = s1 * (d + 16.f * kU) + 4.f * eta, E2 = E1 + s12 * (d + 16.f * kU), E3 = E1 + s13 * (d + 16.f * kU);
+          const bool yes = sv1 > E1 && sv2 < -E2 && sv3 < -E3, no = sv1 < -E1 || sv2 > E2 || sv3 > E3;
+          if (yes) apart = 2.f * fmaxf(E2 * s12 / (sv1 - sv2), E3 * s13 / (sv1 - sv3));
+          if (no) apart = 0.f;
+        }
         if (sv1 >= 0.f && sv2 <= 0.f && sv3 <= 0.f && sv1 - sv2 > 0.f && sv1 - sv3 > 0.f) {
           s2 = __saturatef(__fdividef(sv1, sv1 - sv2));
           s3 = __saturatef(__fdividef(sv1, sv1 - sv3));
@@ -400,7 +421,8 @@ __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned
   const float dmax = fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi));
   if (c1) {
     evals += 4;
-    return fmaxf(dmax, fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])));
+    const float u = fmaxf(dmax, fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])));
+    return kAgree ? __fadd_ru(u, apart) : u;
   }
   // case 2: u3 = min(u3~, min_i h(T, S_i)).  The second term comes from the slots: once it is
   // below l the item is discarded whatever u3~ is (U of a discarded item is not used

@@ -319,12 +319,6 @@ __device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool a
   return how;
 }
 
-__device__ inline double dist_to_tri64(const BvhDev& B, int j, D3 x) {
-  D3 a, b, c;
-  load_tri_d(B.tri64, B.tri32, j, a, b, c);
-  return len(x - closest_on_triangle(x, a, b, c));
-}
-
 // ----------------------------------------------------------------------------- bounds (Section 3.2)
 
 struct VI {
@@ -333,34 +327,6 @@ struct VI {
   int I;
   D3 q;
 };
-
-// Eq. (uexact): the three vertices are nearest to one triangle S; h(T,S) = max_i |v_i - q_i|.
-__device__ inline double ub_exact(const VI t[3]) { return fmax(t[0].d, fmax(t[1].d, t[2].d)); }
-
-// Eq. (u1)
-__device__ inline double ub_u1(const VI t[3]) {
-  double u = INFINITY;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    double e1 = len(t[i].v - t[(i + 1) % 3].v), e2 = len(t[i].v - t[(i + 2) % 3].v);
-    u = fmin(u, fmax(e1, e2) + t[i].d);
-  }
-  return u;
-}
-
-// Eq. (u2): g + max_i d_i with g = R if s - r > 2R, else half the longest edge.
-__device__ inline double ub_u2(const VI t[3]) {
-  double e1 = len(t[1].v - t[2].v), e2 = len(t[2].v - t[0].v), e3 = len(t[0].v - t[1].v);
-  double area = 0.5 * len(cross(t[1].v - t[0].v, t[2].v - t[0].v));
-  double g = 0.5 * fmax(e1, fmax(e2, e3));
-  if (area > 0.0) {
-    double R = e1 * e2 * e3 / (4.0 * area);
-    double s = 0.5 * (e1 + e2 + e3);
-    double r = area / s;
-    if (s - r > 2.0 * R) g = R;
-  }
-  return g + fmax(t[0].d, fmax(t[1].d, t[2].d));
-}
 
 __device__ inline D3 tri_vertex(const BvhDev& B, int j, int slot) {
   if (B.tri64) {
@@ -371,8 +337,63 @@ __device__ inline D3 tri_vertex(const BvhDev& B, int j, int slot) {
   return {v.x, v.y, v.z};
 }
 
-// Kang et al. 2018 bound, Eqs. (Kang2018_case1) and (Kang2018_case2).
-__device__ inline double ub_u3(const BvhDev& B, const VI t[3], unsigned& evals) {
+// Distance from x to triangle j of B, where it may exceed h: an FP32 upper bound of it (pt_hi)
+// first, and the FP64 distance only if that does not settle the comparison.
+__device__ inline void raise_dist(const BvhDev& B, int j, D3 x, double& h, unsigned& evals) {
+  FFP P;
+  P.h = {__double2float_rn(x.x), __double2float_rn(x.y), __double2float_rn(x.z)};
+  P.l = {__double2float_rn(x.x - (double)P.h.x), __double2float_rn(x.y - (double)P.h.y),
+         __double2float_rn(x.z - (double)P.h.z)};
+  const float4* t = B.tri32 + 3 * (size_t)j;
+  // the float forms of B and x, and the FP64 rounding (NearestD::guard)
+  const float guard = __fmaf_ru(0x1p-39f, amax3(P.h), __fadd_ru(__ldg(B.meta), 1e-37f));
+  ++evals;
+  if (__fadd_ru(pt_hi(P, __ldg(t), __ldg(t + 1), __ldg(t + 2)), guard) <= __double2float_rd(h)) return;
+  D3 q;
+  h = fmax(h, sqrt(tri_dist2(B.tri64, B.tri32, j, x, q)));
+}
+
+// Eq. (uexact): the three vertices are nearest to one triangle S; h(T,S) = max_i |v_i - q_i|.
+__device__ inline double ub_exact(const VI t[3]) { return fmax(t[0].d, fmax(t[1].d, t[2].d)); }
+
+// The lengths of T's edges, e[i] opposite vertex i, for u1 and u2.
+struct EdgesD {
+  double e[3];
+  __device__ explicit EdgesD(const VI t[3])
+      : e{len(t[1].v - t[2].v), len(t[2].v - t[0].v), len(t[0].v - t[1].v)} {}
+};
+
+// Eq. (u1)
+__device__ inline double ub_u1(const VI t[3], const EdgesD& E) {
+  return fmin(fmax(E.e[1], E.e[2]) + t[0].d, fmin(fmax(E.e[2], E.e[0]) + t[1].d, fmax(E.e[0], E.e[1]) + t[2].d));
+}
+
+// The bounds below take `cap`, the smallest bound of T so far: where a bound is certain to be
+// at least cap, it may return any value from cap up (it then neither lowers U nor, U being
+// at least l, discards T).
+
+// Eq. (u2): g + max_i d_i with g = R if s - r > 2R, else half the longest edge (g is at least
+// that in either case).
+__device__ inline double ub_u2(const VI t[3], const EdgesD& E, double cap) {
+  double g = 0.5 * fmax(E.e[0], fmax(E.e[1], E.e[2]));
+  const double dmax = fmax(t[0].d, fmax(t[1].d, t[2].d));
+  if (g + dmax > cap * (1.0 + 1e-12)) return INFINITY;
+  double area = 0.5 * len(cross(t[1].v - t[0].v, t[2].v - t[0].v));
+  if (area > 0.0) {
+    double R = E.e[0] * E.e[1] * E.e[2] / (4.0 * area);
+    double s = 0.5 * (E.e[0] + E.e[1] + E.e[2]);
+    double r = area / s;
+    if (s - r > 2.0 * R) g = R;
+  }
+  return g + dmax;
+}
+
+// Kang et al. 2018 bound, Eqs. (Kang2018_case1) and (Kang2018_case2).  own[i] = d(v_i, S_i).
+// Every term is a maximum of point-triangle distances, so a distance is computed in FP64 only
+// where its FP32 upper bound exceeds the maximum so far (raise_dist); a maximum that
+// can no longer lower the minimum it enters is abandoned.  The loops are not unrolled: one
+// copy of the FP64 test per loop keeps the kernel within the instruction cache.
+__device__ inline double ub_u3(const BvhDev& B, const VI t[3], const double own[3], double cap, unsigned& evals) {
   int lone = -1;
   if (!(t[0].I == t[1].I && t[1].I == t[2].I)) {
     if (t[1].I == t[2].I) lone = 0;
@@ -384,6 +405,7 @@ __device__ inline double ub_u3(const BvhDev& B, const VI t[3], unsigned& evals) 
   VI v1 = t[0], v2 = t[1], v3 = t[2];
   if (lone == 1) { v1 = t[1]; v2 = t[2]; v3 = t[0]; }
   else if (lone == 2) { v1 = t[2]; v2 = t[0]; v3 = t[1]; }
+  const double dmax = fmax(own[0], fmax(own[1], own[2]));
   if (lone >= 0 && shared_edge(B, v1.I, v2.I, fs0, fs1, fo, go)) {
     int S1 = v1.I, S2 = v2.I;
     D3 p0 = tri_vertex(B, S1, fs0), e = tri_vertex(B, S1, fs1) - p0;
@@ -403,54 +425,60 @@ __device__ inline double ub_u3(const BvhDev& B, const VI t[3], unsigned& evals) 
         }
       }
     }
-    evals += 7;
-    double hR = fmax(dist_to_tri64(B, S1, v1.v), fmax(dist_to_tri64(B, S1, b1), dist_to_tri64(B, S1, b2)));
-    double hQ = fmax(fmax(dist_to_tri64(B, S2, v3.v), dist_to_tri64(B, S2, b2)),
-                     fmax(dist_to_tri64(B, S2, b1), dist_to_tri64(B, S2, v2.v)));
-    return fmax(hR, hQ);
+    // v1 against S1, v2 and v3 against S2 are the vertices' own; the split points against both
+    double h = dmax;
+#pragma unroll 1
+    for (int k = 0; k < 4 && h < cap; ++k) raise_dist(B, k < 2 ? S1 : S2, (k & 1) ? b2 : b1, h, evals);
+    return h;
   }
-  D3 m[3], bc = (1.0 / 3.0) * (t[0].v + t[1].v + t[2].v);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) m[i] = 0.5 * (t[i].v + t[(i + 1) % 3].v);
-  double ut = 0.0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    int S = t[i].I;
-    double h = fmax(fmax(dist_to_tri64(B, S, t[i].v), dist_to_tri64(B, S, m[i])),
-                    fmax(dist_to_tri64(B, S, bc), dist_to_tri64(B, S, m[(i + 2) % 3])));
-    ut = fmax(ut, h);
-  }
-  double best = INFINITY;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    double h = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) h = fmax(h, dist_to_tri64(B, t[i].I, t[j].v));
+  // min over the triangles of the largest vertex distance to each
+  double best = cap;
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    const int S = k == 0 ? t[0].I : k == 1 ? t[1].I : t[2].I;
+    const D3 x = k == 0 ? t[1].v : k == 1 ? t[2].v : t[0].v, y = k == 0 ? t[2].v : k == 1 ? t[0].v : t[1].v;
+    double h = k == 0 ? own[0] : k == 1 ? own[1] : own[2];
+#pragma unroll 1
+    for (int j = 0; j < 2 && h < best; ++j) raise_dist(B, S, j ? y : x, h, evals);
     best = fmin(best, h);
   }
-  evals += 21;
+  // the quadrilaterals (v_i, m_i, b, m_{i-1}) against S_i
+  const D3 m0 = 0.5 * (t[0].v + t[1].v), m1 = 0.5 * (t[1].v + t[2].v), m2 = 0.5 * (t[2].v + t[0].v),
+           bc = (1.0 / 3.0) * (t[0].v + t[1].v + t[2].v);
+  double ut = dmax;
+#pragma unroll 1
+  for (int k = 0; k < 9 && ut < best; ++k) {
+    const int i = k / 3, j = k % 3;
+    const int S = i == 0 ? t[0].I : i == 1 ? t[1].I : t[2].I;
+    D3 x = bc;
+    if (j == 0) x = i == 0 ? m0 : i == 1 ? m1 : m2;
+    else if (j == 1) x = i == 0 ? m2 : i == 1 ? m0 : m1;
+    raise_dist(B, S, x, ut, evals);
+  }
   return fmin(ut, best);
 }
 
 // Squared max over T of d(., {a, b}), attained at a vertex of T or where an edge of T crosses
-// the bisector plane of a and b (Section 3.2.4).  Squared distances throughout: the one square
-// root is taken by ub_u4 (FP64 square roots are costly on GB300, whose FP64 rate is low).
-__device__ inline double h2_two_points(const VI t[3], D3 a, D3 b) {
+// the bisector plane of a and b (Section 3.2.4), or +inf once it exceeds cap2.  Squared
+// distances throughout: the one square root is taken by ub_u4 (FP64 square roots are costly
+// on GB300, whose FP64 rate is low).
+__device__ inline double h2_two_points(const VI t[3], D3 a, D3 b, double cap2) {
   double h2 = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     D3 ea = t[i].v - a, eb = t[i].v - b;
     h2 = fmax(h2, fmin(dot(ea, ea), dot(eb, eb)));
   }
+  if (h2 > cap2) return INFINITY;
   D3 n = b - a;
   if (dot(n, n) == 0.0) return h2;
   D3 mid = 0.5 * (a + b);
+  const double c[3] = {dot(n, t[0].v - mid), dot(n, t[1].v - mid), dot(n, t[2].v - mid)};
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    D3 x0 = t[i].v, x1 = t[(i + 1) % 3].v;
-    double c0 = dot(n, x0 - mid), c1 = dot(n, x1 - mid);
+    const double c0 = c[i], c1 = c[(i + 1) % 3];
     if (((c0 <= 0.0 && c1 >= 0.0) || (c0 >= 0.0 && c1 <= 0.0)) && c0 != c1) {
-      D3 x = x0 + (c0 / (c0 - c1)) * (x1 - x0);
+      D3 x = t[i].v + (c0 / (c0 - c1)) * (t[(i + 1) % 3].v - t[i].v);
       D3 ea = x - a, eb = x - b;
       h2 = fmax(h2, fmin(dot(ea, ea), dot(eb, eb)));
     }
@@ -459,7 +487,7 @@ __device__ inline double h2_two_points(const VI t[3], D3 a, D3 b) {
 }
 
 // Eq. (bound_u4)
-__device__ inline double ub_u4(const VI t[3]) {
+__device__ inline double ub_u4(const VI t[3], double cap) {
   D3 e0 = t[0].v - t[1].v, e1 = t[1].v - t[2].v, e2 = t[2].v - t[0].v;
   double l0 = dot(e0, e0), l1 = dot(e1, e1), l2 = dot(e2, e2);
   int k = 0;
@@ -469,24 +497,31 @@ __device__ inline double ub_u4(const VI t[3]) {
   D3 q2 = t[0].q, q3 = t[1].q, q1 = t[2].q;  // shortest edge v1v2 (k = 0)
   if (k == 1) { q2 = t[1].q; q3 = t[2].q; q1 = t[0].q; }
   else if (k == 2) { q2 = t[2].q; q3 = t[0].q; q1 = t[1].q; }
-  return sqrt(fmin(h2_two_points(t, q1, q2), h2_two_points(t, q1, q3)));
+  double h2 = INFINITY;
+  const double cap2 = cap * cap * (1.0 + 1e-12);
+#pragma unroll 1
+  for (int j = 0; j < 2; ++j) h2 = fmin(h2, h2_two_points(t, q1, j ? q3 : q2, fmin(cap2, h2)));
+  return sqrt(h2);
 }
 
-// UpperBound(T, l) of Section 4.
-__device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], double l, const uint8_t* order, int nb,
-                                       int& code, unsigned& evals) {
+// UpperBound(T, l) of Section 4; own[i] = d(v_i, S_i).  With `full`, every bound is evaluated
+// in full (a discarded T then returns the deciding bound's own value).
+__device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const double own[3], double l,
+                                       const uint8_t* order, int nb, bool full, int& code, unsigned& evals) {
   if (t[0].I == t[1].I && t[1].I == t[2].I) {
     code = 0;
     return ub_exact(t);
   }
   double U = INFINITY;
+  const EdgesD E(t);
   for (int k = 0; k < nb; ++k) {
     double u;
+    const double cap = full ? INFINITY : U;
     switch (order[k]) {
-      case 1: u = ub_u1(t); break;
-      case 2: u = ub_u2(t); break;
-      case 3: u = ub_u3(B, t, evals); break;
-      default: u = ub_u4(t); break;
+      case 1: u = ub_u1(t, E); break;
+      case 2: u = ub_u2(t, E, cap); break;
+      case 3: u = ub_u3(B, t, own, cap, evals); break;
+      default: u = ub_u4(t, cap); break;
     }
     if (u < l) {
       code = order[k];
@@ -503,6 +538,9 @@ __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], double l,
 #ifndef HD_FP64_BOUND_REGS
 #define HD_FP64_BOUND_REGS 128
 #endif
+#ifndef HD_FP64_PAPER_REGS
+#define HD_FP64_PAPER_REGS 96
+#endif
 
 struct PolicyD {
   using Vtx = VtxD;
@@ -512,6 +550,7 @@ struct PolicyD {
   static constexpr int kCoopBlocks = HD_COOP_MIN_BLOCKS_D;  // resident blocks per SM of the cooperative traversal
   static constexpr int kLongBudget = HD_LONG_BUDGET_D;      // triangle tests of a lane before the hand-off
   static constexpr int kBoundRegs = HD_FP64_BOUND_REGS;  // register cap of the UpperBound kernels
+  static constexpr int kPaperRegs = HD_FP64_PAPER_REGS;  // ... of their paper-order instantiation
 
   // Nearest triangle of v.  Called by every lane of the warp (the traversal votes over the
   // full warp); lanes with active == false only vote and leave v untouched.  With `over`
@@ -600,7 +639,6 @@ struct PolicyD {
   __device__ static D3 out_foot(const Vtx& v) { return {v.qx, v.qy, v.qz}; }
   static double slack(double) { return 0.0; }
   __device__ static double ut_down(double x) { return x; }
-  __device__ static double bound_u4(const Vtx&, const Vtx&, const Vtx&, const RunParams&, double) { return INFINITY; }
   __device__ static D3 exact_pos(const Vtx& v) { return {v.x, v.y, v.z}; }
   __device__ static bool promote(const Vtx&, const Vtx&, const Vtx&, double, double) { return false; }
   __device__ static void set_pos_f(Vtx& v, float x, float y, float z) { set_pos(v, x, y, z); }
@@ -629,15 +667,123 @@ struct PolicyD {
     m.tri = -2;
     m.hint = a.tri;
   }
-  __device__ static UT upper_bound(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, double l, float,
+  // The FP32 filter of the UpperBound kernels.  An item's vertices as float pairs, their
+  // distances rounded up:
+  __device__ static void vertices_m(const Vtx& a, const Vtx& b, const Vtx& c, VM t[3]) {
+    auto one = [](const Vtx& v) {
+      VM m;
+      m.p.h = {__double2float_rn(v.x), __double2float_rn(v.y), __double2float_rn(v.z)};
+      m.p.l = {__double2float_rn(v.x - (double)m.p.h.x), __double2float_rn(v.y - (double)m.p.h.y),
+               __double2float_rn(v.z - (double)m.p.h.z)};
+      m.dhi = __double2float_ru(v.d);
+      m.I = v.tri;
+      m.q = {0.f, 0.f, 0.f};
+      m.qerr = 0.f;
+      return m;
+    };
+    t[0] = one(a);
+    t[1] = one(b);
+    t[2] = one(c);
+  }
+  // An FP32 bound below this discards the item, as the FP64 bound then also does (it lies
+  // below the FP32 bound up to its own rounding): l less 2^-14 of it, the slack, the distance
+  // of B's float vertices from its own, and the float pairs' rounding.
+  __device__ static float filter_limit(const BvhDev& B, const VM t[3], float lf, const RunParams& rp) {
+    const float pmax = fmaxf(amax3(t[0].p.h), fmaxf(amax3(t[1].p.h), amax3(t[2].p.h)));
+    const float guard = __fadd_ru(__fmaf_ru(0x1p-38f, pmax, __fadd_ru(__ldg(B.meta), 1e-37f)), rp.slack_f);
+    return __fsub_rd(__fmul_rd(lf, 1.f - 0x1p-14f), guard);
+  }
+  // The cascade's part in the UpperBound kernels: the exact case, and the items that certified
+  // FP32 bounds u1..u3 discard.  Every other item is left (kDeferU4, U = +inf) to the pass
+  // that bounds them in FP64 with every lane of a warp on an item of its own: about one
+  // item in ten is left, and each would hold its whole warp for the FP64 cascade.  (Inlined
+  // 21 times and run by every item, that cascade also outgrew the instruction cache: 45
+  // cycles of instruction fetch per instruction issued.)  Torus pair in FP64: the bounds of
+  // 200,000 faces and 138,480 children 4.59 -> 0.47 ms.
+  __device__ static UT upper_bound_paper(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, double,
+                                         float lf, const RunParams& rp, int& code, Counters& cnt) {
+    UT U;
+    float u12;
+    if (!paper_cheap(B, a, b, c, lf, rp, &U, &code, &u12)) return U;
+    return paper_u3(B, a, b, c, lf, rp, u12, code, cnt);
+  }
+  __device__ static bool paper_cheap(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf,
+                                     const RunParams& rp, UT* U, int* code, float* u12) {
+    if (a.tri == b.tri && b.tri == c.tri) {
+      *code = 0;
+      *U = fmax(a.d, fmax(b.d, c.d)) + rp.slack;
+      return false;
+    }
+    VM t[3];
+    vertices_m(a, b, c, t);
+    const float lim = filter_limit(B, t, lf, rp);
+    const EdgesM E(t);
+    const float u1 = ubm_u1(t, E);
+    if (u1 < lim) {
+      *code = 1;
+      *U = (UT)u1;
+      return false;
+    }
+    const float u2 = ubm_u2(t, E);
+    if (u2 < lim) {
+      *code = 2;
+      *U = (UT)u2;
+      return false;
+    }
+    *u12 = fminf(u1, u2);
+    return true;
+  }
+  __device__ static UT paper_u3(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf, const RunParams& rp,
+                                float, int& code, Counters& cnt) {
+    VM t[3];
+    vertices_m(a, b, c, t);
+    const float lim = filter_limit(B, t, lf, rp);
+    if (lim > 0.f) {
+      const float u3 = ubm_u3<true>(B, t, lim, cnt.evals);
+      if (u3 < lim) {
+        code = 3;
+        return (UT)u3;
+      }
+    }
+    code = kDeferU4;
+    return INFINITY;
+  }
+  // The same for a cascade in any order.
+  __device__ static UT upper_bound(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, double, float lf,
                                    const RunParams& rp, int& code, Counters& cnt) {
-    VI t[3] = {{{a.x, a.y, a.z}, a.d, a.tri, {a.qx, a.qy, a.qz}},
-               {{b.x, b.y, b.z}, b.d, b.tri, {b.qx, b.qy, b.qz}},
-               {{c.x, c.y, c.z}, c.d, c.tri, {c.qx, c.qy, c.qz}}};
+    if (a.tri == b.tri && b.tri == c.tri) {
+      code = 0;
+      return fmax(a.d, fmax(b.d, c.d)) + rp.slack;
+    }
+    VM t[3];
+    vertices_m(a, b, c, t);
+    const float lim = filter_limit(B, t, lf, rp);
+    if (lim > 0.f) {
+      const EdgesM E(t);
+      for (int k = 0; k < rp.n_bounds; ++k) {
+        const int o = rp.order[k];
+        if (o == 4) continue;
+        const float u = o == 1 ? ubm_u1(t, E) : o == 2 ? ubm_u2(t, E) : ubm_u3<true>(B, t, lim, cnt.evals);
+        if (u < lim) {
+          code = o;
+          return (UT)u;
+        }
+      }
+    }
+    code = kDeferU4;
+    return INFINITY;
+  }
+  // The pass over the items left: the whole cascade in FP64, clamped to what U holds.
+  __device__ static void bound_deferred(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, double l, UT,
+                                        const RunParams& rp, UT& U, int& code, Counters& cnt) {
+    const VI t[3] = {{{a.x, a.y, a.z}, a.d, a.tri, {a.qx, a.qy, a.qz}},
+                     {{b.x, b.y, b.z}, b.d, b.tri, {b.qx, b.qy, b.qz}},
+                     {{c.x, c.y, c.z}, c.d, c.tri, {c.qx, c.qy, c.qz}}};
+    const double own[3] = {a.d, b.d, c.d};
     // slack is 0 in a pure FP64 run; in the certification phase of a MIXED run it is the
     // margin that covers the double rounding
-    double U = upper_bound_d(B, t, l - rp.slack, rp.order, rp.n_bounds, code, cnt.evals);
-    return U + rp.slack;
+    const double u = upper_bound_d(B, t, own, l - rp.slack, rp.order, rp.n_bounds, false, code, cnt.evals) + rp.slack;
+    U = fmin(U, u);
   }
 };
 

@@ -119,7 +119,7 @@ struct RunState {
   int overflow;                  // next frontier or split list ran out of room
   int err;                       // traversal stack overflow and similar
   int n_promote;                 // MIXED items handed to the FP64 phase
-  int n_u4;                      // MIXED items whose u4 is evaluated in the separate u4 pass
+  int n_u4;                      // items left to the second pass of the bounds
   unsigned long long upro_bits;  // max U of those items (double bits)
   unsigned long long evals, box_tests, queries, retired, escalations, leaf_tests;
   unsigned long long discards[6];
@@ -237,7 +237,7 @@ struct RunParams {
   uint8_t order[4];
   int n_bounds;
   float slack_f;  // slack rounded up to float
-  int defer_u4;   // MIXED: a trailing u4 is evaluated in the separate u4 pass
+  int defer_u4;   // a trailing u4 is evaluated in the second pass of the bounds
   int parent_clamp;  // children's U is clamped to their parent's U
   const DynParams* dyn;  // if set, eps / slack / slack_f are taken from here on the device
 };
@@ -251,7 +251,7 @@ __device__ inline RunParams with_dyn(RunParams rp) {
   return rp;
 }
 
-// UpperBound result code: u4 still to be evaluated by the u4 pass (MIXED)
+// UpperBound result code: left to the second pass of the bounds (MIXED: u4; FP64: the cascade)
 constexpr int kDeferU4 = 6;
 
 // Per-thread statistics, flushed with one atomic per warp.

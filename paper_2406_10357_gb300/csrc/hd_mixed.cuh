@@ -322,7 +322,6 @@ __device__ inline FFP pair_add(const FFP& a, const FFP& b) {
 __device__ inline F3 pair_f(const FFP& a) {  // h + l rounded: within u |h + l| per component
   return {__fadd_rn(a.h.x, a.l.x), __fadd_rn(a.h.y, a.l.y), __fadd_rn(a.h.z, a.l.z)};
 }
-__device__ inline float sum1(F3 a) { return __fadd_ru(__fadd_ru(fabsf(a.x), fabsf(a.y)), fabsf(a.z)); }
 
 // Upper bound of the length of the exact vector whose float-pair form rounds to d: each
 // component of d is within u |d_c| + 3T of it (two differences of pairs and one more pair
@@ -511,13 +510,16 @@ struct PolicyM {
   // vertices (2^-48 relative per level, at most 60 levels) and the double rounding of u4
   static double slack(double amax) { return ldexp(amax, -40); }
   __device__ static float ut_down(double x) { return __double2float_rd(x); }
-  // the u4 pass: Eq. (bound_u4) for one item (certified FP32), plus the slack.  The item's
-  // bound so far (the last argument) is not needed.
-  __device__ static float bound_u4(const Vtx& a, const Vtx& b, const Vtx& c, const RunParams& rp, float) {
+  // the pass over the items left: u4, Eq. (bound_u4), for one item (certified FP32), plus the
+  // slack; U holds the item's bound so far.
+  __device__ static void bound_deferred(const BvhDev&, const Vtx& a, const Vtx& b, const Vtx& c, double, float lo,
+                                        const RunParams& rp, float& U, int& code, Counters&) {
     const VM t[3] = {{pos(a), a.dhi, a.tri, {a.qx, a.qy, a.qz}, a.qerr},
                      {pos(b), b.dhi, b.tri, {b.qx, b.qy, b.qz}, b.qerr},
                      {pos(c), c.dhi, c.tri, {c.qx, c.qy, c.qz}, c.qerr}};
-    return __fadd_ru(ubm_u4(t, rp.slack_f), rp.slack_f);
+    const float u = __fadd_ru(ubm_u4(t, rp.slack_f), rp.slack_f);
+    code = u < lo ? 4 : 5;
+    if (u < lo || u < U) U = u;
   }
 
   __device__ static FFP pos(const Vtx& v) { return {{v.hx, v.hy, v.hz}, {v.lx, v.ly, v.lz}}; }
@@ -698,8 +700,8 @@ struct PolicyM {
   // full warps: paper_cheap runs the exact case, u1 and u2; it returns true when u3 is still
   // needed (U so far in *u12), else the result in *U and *code as upper_bound_paper.
   // paper_u3 then finishes such an item; together they give upper_bound_paper's values.
-  __device__ static bool paper_cheap(const Vtx& a, const Vtx& b, const Vtx& c, float lf, const RunParams& rp,
-                                     float* U, int* code, float* u12) {
+  __device__ static bool paper_cheap(const BvhDev&, const Vtx& a, const Vtx& b, const Vtx& c, float lf,
+                                     const RunParams& rp, float* U, int* code, float* u12) {
     const VM t[3] = {{pos(a), a.dhi, a.tri, {0.f, 0.f, 0.f}, 0.f},
                      {pos(b), b.dhi, b.tri, {0.f, 0.f, 0.f}, 0.f},
                      {pos(c), c.dhi, c.tri, {0.f, 0.f, 0.f}, 0.f}};

@@ -57,3 +57,34 @@ def test_nearest_fp64_filtered(hd, orc, n, scale, shift, vtype, leaf):
         dd, _ = orc.point_triangle(P[i], *T[idx[i]])
         assert abs(dd - do[i]) <= 1e-12 * C
     assert np.max(np.abs(np.linalg.norm((P - foot) / scale, axis=1) * scale - d)) <= 1e-12 * C
+
+
+def _perturbed_copy(nu, nv, sigma, scale, shift, dtype):
+    """A torus and a copy of it moved along its normals: A's edges follow B's, so vertices of A's
+    sub-triangles lie close to u3's bisecting planes."""
+    P, F, N = mg.torus(1.0, 0.3, nu, nv)
+    g = mg.stream(11, nu)
+    VA, VB = P * scale + shift, (P + N * g.normal(len(P), sigma)[:, None]) * scale + shift
+    return VA.astype(dtype), F, VB.astype(dtype), F.copy()
+
+
+@pytest.mark.parametrize("nu,nv,sigma,tol", [(3, 3, 1e-1, 1e-4), (16, 9, 1e-2, 1e-5), (24, 11, 1e-3, 1e-5)])
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1.0, 1e4), (1e-25, 0.0), (1e25, 0.0)])
+@pytest.mark.parametrize("order", [(1, 2, 3, 4), (3, 1), (4, 3)])
+def test_bracket_fp64_filtered(hd, orc, nu, nv, sigma, tol, scale, shift, order):
+    """The bracket of a pair whose bounds the filter decides meets the oracle's and a tighter
+    one's, alone and in a batch; the two runs split the same sub-triangles.  Both sides hold h
+    up to their rounding, 1e-12 of the largest coordinate."""
+    VA, FA, VB, FB = _perturbed_copy(nu, nv, sigma, scale, shift, np.float64)
+    o = hd.hd_options_default(tol_mode=hd.HD_TOL_REL, bound_order=order)
+    bvh = hd.hd_build_B(VB, FB)
+    r = hd.hd_hausdorff(bvh, VA, FA, tol, o)
+    rb, _ = hd.hd_hausdorff_batched([bvh, bvh], [(VA, FA), (VA, FA)], tol, o)
+    ro = orc.hausdorff(VA, FA, VB, FB, tol, 1)
+    rt = orc.hausdorff(VA, FA, VB, FB, tol / 10, 1)
+    eps, C = r["stats"]["eps_abs"], max(np.abs(VA).max(), np.abs(VB).max())
+    for x in (r, rb):
+        assert x["status"] == hd.HD_OK and x["upper"] - x["lower"] <= eps * (1 + 1e-12) + 1e-12 * C
+        for y in (ro, rt):
+            assert max(x["lower"], y["lower"]) <= min(x["upper"], y["upper"]) + 1e-12 * C
+    assert r["stats"]["splits"] == rb["stats"]["splits"] and r["stats"]["rounds"] == rb["stats"]["rounds"]
