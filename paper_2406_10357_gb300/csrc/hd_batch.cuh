@@ -88,9 +88,7 @@ __device__ inline int find_pair(const int* base, int np, int g) {
 // The pair all lanes with a pair (>= 0) share, -1 if no lane has one, -2 if they differ.
 // Every lane of the warp must call it.
 __device__ inline int warp_pair(int pair) {
-  const int key = pair >= 0 ? pair : INT_MAX;
-  int m = key;
-  for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int m = __reduce_min_sync(0xffffffffu, pair >= 0 ? pair : INT_MAX);
   if (m == INT_MAX) return -1;
   return __all_sync(0xffffffffu, pair < 0 || pair == m) ? m : -2;
 }
@@ -110,87 +108,152 @@ __device__ inline PairLevel<P> pair_level(const BatchCtx& x, int p) {
   return PairLevel<P>{rp, Level<P>{l, __double2float_rd(l), Thresholds<P>(l, rp.eps)}};
 }
 
-// Work counters of one lane for pair `pair` (-1: none), flushed per batch of 32.  Every lane
-// of the warp must call it.
-__device__ inline void flush_counters_pair(RunState* sts, int pair, const Counters& c, bool long_pass = false) {
-  const int u = warp_pair(pair);
-  if (u >= 0) {
-    flush_counters(sts + u, c, long_pass);
-    return;
-  }
-  if (u == -1 || pair < 0) return;
-  RunState* st = sts + pair;
-  if (c.evals + c.leaf) atomicAdd(&st->evals, (unsigned long long)(c.evals + c.leaf));
-  if (c.leaf) atomicAdd(&st->leaf_tests, (unsigned long long)c.leaf);
-  if (c.boxes) atomicAdd(&st->box_tests, (unsigned long long)c.boxes);
-  if (c.escalations) atomicAdd(&st->escalations, (unsigned long long)c.escalations);
-  if (c.nodes) atomicAdd(&st->node_visits, (unsigned long long)c.nodes);
-  if (long_pass && c.nodes) atomicAdd(&st->long_node_visits, (unsigned long long)c.nodes);
-  if (long_pass && c.leaf) atomicAdd(&st->long_leaf_tests, (unsigned long long)c.leaf);
-  if (c.err) atomicExch(&st->err, 1);
-}
-
-// Lower bound and query count of one lane for its pair.  Every lane must call it.  l stays
-// non-negative (a certified vertex distance less its slack can be below 0), which the atomic
-// maximum on its bits needs.
-__device__ inline void flush_lower_pair(RunState* sts, int pair, double lmax, int nq, bool long_pass) {
-  lmax = fmax(lmax, 0.0);
-  const int u = warp_pair(pair);
-  if (u >= 0) {
-    const double m = warp_max(pair >= 0 ? lmax : 0.0);
-    const unsigned long long q = warp_sum((unsigned long long)(pair >= 0 ? nq : 0));
-    if ((threadIdx.x & 31) == 0) {
-      atomic_max_nonneg(&sts[u].l_bits, m);
-      if (q) atomicAdd(&sts[u].queries, q);
-      if (q && long_pass) atomicAdd(&sts[u].long_queries, q);
-    }
-    return;
-  }
-  if (u == -1 || pair < 0) return;
-  atomic_max_nonneg(&sts[pair].l_bits, lmax);
-  if (nq) atomicAdd(&sts[pair].queries, (unsigned long long)nq);
-  if (nq && long_pass) atomicAdd(&sts[pair].long_queries, (unsigned long long)nq);
-}
-
-// Outcome of one lane's item for its pair (the Tally of a single run, one item at a time,
-// plus the pair's frontier count), flushed per batch of 32.  Every lane must call it.
+// What one lane adds to its pair's state in a batch of 32 items: its work counters, a lower
+// bound, its queries, and an item's outcome.
 template <class P>
-struct PairTally {
+struct PairDelta {
+  Counters c;
+  double l = 0.0;
+  int nq = 0;
   int discard = -1;  // deciding bound of a discard (0..5), -1 none
   int retired = 0, kept = 0;
   typename P::UT uret = 0, umax = 0;
 };
+
+// The sums and maxima of several batches of one pair, per warp (shared memory), added to the
+// pair's state when the warp's batches move on to another pair.  Batches come in the order of
+// the queue, in which a pair's items lie together, so most batches of a warp belong to the
+// pair of the batch before.  With the sums made by shuffles and added to the pair's state
+// after every batch, lane by lane where two pairs meet in one, those atomics were what the
+// batched kernels waited for: all warps add to the few pairs the queue is at, so one slice of
+// the L2 took most of the traffic (83% busy, 8% on average).  In the fourth round of 24 pairs
+// (1K to 200K triangles) the query kernel went from 1.65 to 0.82 ms, the u4 pass from 0.40 to
+// 0.13 ms, the select from 0.28 to 0.15 ms.
+struct PairAcc {
+  unsigned long long l, uret, umax;  // bits of non-negative doubles
+  unsigned evals, leaf, boxes, escalations, nodes, nq, retired, kept;
+  unsigned discards[6];
+  int pair;  // -1: empty
+};
+constexpr int kMaxWarps = 32;  // warps of a block
+
+__device__ inline void acc_reset(PairAcc& a, int pair) {
+  a.l = a.uret = a.umax = 0ull;
+  a.evals = a.leaf = a.boxes = a.escalations = a.nodes = a.nq = a.retired = a.kept = 0u;
+  for (int k = 0; k < 6; ++k) a.discards[k] = 0u;
+  a.pair = pair;
+}
+
+// Adds `a` to the state of its pair (one lane).
+__device__ inline void acc_apply(RunState* sts, const PairAcc& a, bool long_pass) {
+  if (a.pair < 0) return;
+  RunState* st = sts + a.pair;
+  auto add = [](unsigned long long* p, unsigned v) {
+    if (v) atomicAdd(p, (unsigned long long)v);
+  };
+  if (a.l) atomicMax(&st->l_bits, a.l);
+  add(&st->queries, a.nq);
+  add(&st->evals, a.evals + a.leaf);
+  add(&st->leaf_tests, a.leaf);
+  add(&st->box_tests, a.boxes);
+  add(&st->escalations, a.escalations);
+  add(&st->node_visits, a.nodes);
+  if (long_pass) {
+    add(&st->long_queries, a.nq);
+    add(&st->long_node_visits, a.nodes);
+    add(&st->long_leaf_tests, a.leaf);
+  }
+  for (int k = 0; k < 6; ++k) add(&st->discards[k], a.discards[k]);
+  if (a.retired) {
+    add(&st->retired, a.retired);
+    atomicMax(&st->uret_bits, a.uret);
+  }
+  if (a.kept) {
+    atomicAdd(&st->n_next, (int)a.kept);
+    atomicMax(&st->umax_bits, a.umax);
+  }
+}
+
+// Largest non-negative value over the lanes of group g (called by those lanes), as the bits
+// of a double.
+__device__ inline unsigned long long group_max(unsigned g, double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = __reduce_max_sync(g, (unsigned)(b >> 32));
+  const unsigned lo = __reduce_max_sync(g, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+__device__ inline unsigned long long group_max(unsigned g, float v) {
+  return (unsigned long long)__double_as_longlong((double)__uint_as_float(__reduce_max_sync(g, __float_as_uint(v))));
+}
+
+// Adds the lanes' deltas to their pairs.  Every lane of the warp must call it (pair -1:
+// nothing to add); `a` is the warp's accumulator.  l stays non-negative (a certified vertex
+// distance less its slack can be below 0), which the maximum on its bits needs.
 template <class P>
-__device__ inline void flush_tally_pair(RunState* sts, int pair, const PairTally<P>& t) {
-  const int u = warp_pair(pair);
-  if (u >= 0) {
-    Tally<P> w;
-    const bool on = pair >= 0;
-    w.d0 = on && t.discard == 0;
-    w.d1 = on && t.discard == 1;
-    w.d2 = on && t.discard == 2;
-    w.d3 = on && t.discard == 3;
-    w.d4 = on && t.discard == 4;
-    w.d5 = on && t.discard == 5;
-    w.retired = on ? t.retired : 0;
-    w.uret = on ? t.uret : 0;
-    w.umax = on ? t.umax : 0;
-    flush_tally(sts + u, w);
-    const unsigned long long k = warp_sum((unsigned long long)(on ? t.kept : 0));
-    if ((threadIdx.x & 31) == 0 && k) atomicAdd(&sts[u].n_next, (int)k);
-    return;
+__device__ inline void acc_batch(PairAcc& a, RunState* sts, int pair, const PairDelta<P>& d, bool long_pass = false) {
+  const int lane = threadIdx.x & 31;
+  if (d.c.err && pair >= 0) atomicExch(&sts[pair].err, 1);
+  unsigned left = __ballot_sync(0xffffffffu, pair >= 0);
+  while (left) {  // one pair of the warp at a time (uniform)
+    const int p = __shfl_sync(0xffffffffu, pair, __ffs(left) - 1);
+    const unsigned g = __ballot_sync(0xffffffffu, pair == p);
+    left &= ~g;
+    if (a.pair != p) {  // uniform: every lane reads the same value
+      __syncwarp();
+      if (lane == 0) {
+        acc_apply(sts, a, long_pass);
+        acc_reset(a, p);
+      }
+      __syncwarp();
+    }
+    if (pair == p) {
+      const bool first = lane == __ffs(g) - 1;
+      auto sum = [g, first](unsigned& to, unsigned v) {
+        const unsigned s = __reduce_add_sync(g, v);
+        if (first) to += s;
+      };
+      sum(a.evals, d.c.evals);
+      sum(a.leaf, d.c.leaf);
+      sum(a.boxes, d.c.boxes);
+      sum(a.nodes, d.c.nodes);
+      if (__any_sync(g, d.c.escalations != 0)) sum(a.escalations, d.c.escalations);
+      if (__any_sync(g, d.nq != 0)) {
+        sum(a.nq, (unsigned)d.nq);
+        const unsigned long long l = group_max(g, fmax(d.l, 0.0));
+        if (first && l > a.l) a.l = l;
+      }
+      if (__any_sync(g, d.discard >= 0)) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const unsigned m = __ballot_sync(g, d.discard == k);
+          if (first) a.discards[k] += __popc(m);
+        }
+      }
+      if (__any_sync(g, d.retired != 0)) {
+        sum(a.retired, (unsigned)d.retired);
+        const unsigned long long u = group_max(g, fmax(d.uret, typename P::UT(0)));
+        if (first && u > a.uret) a.uret = u;
+      }
+      if (__any_sync(g, d.kept != 0)) {
+        sum(a.kept, (unsigned)d.kept);
+        const unsigned long long u = group_max(g, fmax(d.umax, typename P::UT(0)));
+        if (first && u > a.umax) a.umax = u;
+      }
+    }
+    __syncwarp();
   }
-  if (u == -1 || pair < 0) return;
-  RunState* st = sts + pair;
-  if (t.discard >= 0) atomicAdd(&st->discards[t.discard], 1ull);
-  if (t.retired) {
-    atomicAdd(&st->retired, 1ull);
-    atomic_max_nonneg(&st->uret_bits, (double)t.uret);
-  }
-  if (t.kept) {
-    atomicAdd(&st->n_next, 1);
-    atomic_max_nonneg(&st->umax_bits, (double)t.umax);
-  }
+}
+
+// The warp's accumulator, empty, and its last addition.  Every lane must call both.
+__device__ inline PairAcc& acc_begin(PairAcc* s_acc) {
+  PairAcc& a = s_acc[threadIdx.x >> 5];
+  if ((threadIdx.x & 31) == 0) acc_reset(a, -1);
+  __syncwarp();
+  return a;
+}
+__device__ inline void acc_end(PairAcc& a, RunState* sts, bool long_pass = false) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) acc_apply(sts, a, long_pass);
 }
 
 // Discard / retire / keep one bounded item of pair p (Section 3.1: discard when U < l); a
@@ -198,7 +261,7 @@ __device__ inline void flush_tally_pair(RunState* sts, int pair, const PairTally
 template <class P>
 __device__ inline void classify_pair(BatchState* bs, const typename P::Item& it, int p, const Thresholds<P>& th,
                                      int code, typename P::Item* next, int* next_pair, int next_cap,
-                                     typename P::Item* u4list, int* u4_pair, PairTally<P>& ty) {
+                                     typename P::Item* u4list, int* u4_pair, PairDelta<P>& ty) {
   if (code == kDeferU4) {
     const int j = warp_slot(&bs->n_u4);
     if (j < next_cap) {
@@ -338,9 +401,11 @@ static __global__ void k_batch_prep_finish(BatchCtx x, unsigned long long* boxes
 template <class P>
 __global__ void HD_QUERY_REGS k_batch_query(BatchCtx x, typename P::Vtx* pool, const int* vpair, LongList ll,
                                             bool round_midpoints) {
+  __shared__ PairAcc s_acc[kMaxWarps];
   grid_dep_wait();
   grid_dep_launch();
   BatchState* bs = x.bs;
+  PairAcc& acc = acc_begin(s_acc);
   int beg = 0, count = x.nV;
   if (round_midpoints) {
     if (bs->stop) return;  // uniform over the grid
@@ -359,12 +424,10 @@ __global__ void HD_QUERY_REGS k_batch_query(BatchCtx x, typename P::Vtx* pool, c
       p = vpair[beg + t];
     }
     const bool q = active && p >= 0 && v.tri != -1;
-    Counters c;
+    PairDelta<P> d;
     bool over = false;
     const BvhDev B = x.pd[q ? p : 0].B;
-    P::query(B, v, c, q, ll.idx ? P::kLongBudget : INT_MAX, &over);
-    double lmax = 0.0;
-    int nq = 0;
+    P::query(B, v, d.c, q, ll.idx ? P::kLongBudget : INT_MAX, &over);
     if (q) {
       pool[beg + t] = v;
       if (over) {
@@ -372,14 +435,13 @@ __global__ void HD_QUERY_REGS k_batch_query(BatchCtx x, typename P::Vtx* pool, c
         if (j < ll.cap) ll.idx[j] = beg + t;
         else atomicExch(&bs->overflow, 1);
       } else {
-        lmax = P::lower(v) - x.dyn[p].slack;
-        nq = 1;
+        d.l = P::lower(v) - x.dyn[p].slack;
+        d.nq = 1;
       }
     }
-    const int fp = q ? p : -1;
-    flush_lower_pair(x.sts, fp, lmax, nq, false);
-    flush_counters_pair(x.sts, fp, c);
+    acc_batch(acc, x.sts, q ? p : -1, d);
   }
+  acc_end(acc, x.sts);
 }
 
 // The handed-off queries, one warp each (traverse_coop), with their pair's BVH.
@@ -388,10 +450,12 @@ __global__ void __launch_bounds__(32 * kCoopWarps, P::kCoopBlocks)
     k_batch_query_long(BatchCtx x, typename P::Vtx* pool, const int* vpair, LongList ll, bool round_midpoints) {
   __shared__ unsigned s_code[kCoopWarps * kCoopStack];
   __shared__ float s_e[kCoopWarps * kCoopStack];
+  __shared__ PairAcc s_acc[kCoopWarps];
   grid_dep_wait();
   grid_dep_launch();
   BatchState* bs = x.bs;
   if (round_midpoints && bs->stop) return;
+  PairAcc& acc = acc_begin(s_acc);
   const int n = min(bs->n_long, ll.cap);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (;;) {
@@ -402,12 +466,16 @@ __global__ void __launch_bounds__(32 * kCoopWarps, P::kCoopBlocks)
     const int k = ll.idx[i];
     const int p = vpair[k];
     typename P::Vtx v = pool[k];
-    Counters c;
-    P::query_coop(x.pd[p].B, v, c, s_code + w * kCoopStack, s_e + w * kCoopStack);
-    if (lane == 0) pool[k] = v;
-    flush_lower_pair(x.sts, lane == 0 ? p : -1, P::lower(v) - x.dyn[p].slack, 1, true);
-    flush_counters_pair(x.sts, p, c, true);
+    PairDelta<P> d;
+    P::query_coop(x.pd[p].B, v, d.c, s_code + w * kCoopStack, s_e + w * kCoopStack);
+    if (lane == 0) {
+      pool[k] = v;
+      d.l = P::lower(v) - x.dyn[p].slack;
+      d.nq = 1;
+    }
+    acc_batch(acc, x.sts, p, d, true);
   }
+  acc_end(acc, x.sts, true);
 }
 
 // ----------------------------------------------------------------------------- bounds
@@ -431,6 +499,8 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
                                          int* u4_pair, BatchRebinEntry* q, Make make) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
+  __shared__ PairAcc s_acc[kMaxWarps];
+  PairAcc& acc = acc_begin(s_acc);
   int qn = 0;
   bool more = true;
   while (more || qn > 0) {
@@ -445,7 +515,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
         typename P::Item it;
         float up = INFINITY;
         int p = -1;
-        PairTally<P> ty;
+        PairDelta<P> ty;
         if (t < count) p = make(t, it, up);
         if (p >= 0) {
           const PairLevel<P> pl = pair_level<P>(x, p);
@@ -460,7 +530,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
             classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
           }
         }
-        flush_tally_pair<P>(x.sts, need ? -1 : p, ty);
+        acc_batch(acc, x.sts, need ? -1 : p, ty);
         const unsigned m = __ballot_sync(0xffffffffu, need);
         if (need) q[qn + __popc(m & lt)] = e;
         qn += __popc(m);
@@ -470,8 +540,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
     if (qn >= 32 || (!more && qn > 0)) {
       const int take = min(qn, 32);
       int p = -1;
-      Counters cnt;
-      PairTally<P> ty;
+      PairDelta<P> ty;
       if (lane < take) {
         const BatchRebinEntry e = q[qn - take + lane];
         p = e.pair;
@@ -482,16 +551,16 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
         const PairLevel<P> pl = pair_level<P>(x, p);
         int code;
         const typename P::UT U =
-            P::paper_u3(x.pd[p].B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], pl.lv.lf, pl.rp, e.u12, code, cnt);
+            P::paper_u3(x.pd[p].B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], pl.lv.lf, pl.rp, e.u12, code, ty.c);
         it.U = e.up < U ? e.up : U;
         classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
       }
       qn -= take;
       __syncwarp();  // the entries taken are read before new ones overwrite them
-      flush_counters_pair(x.sts, p, cnt);
-      flush_tally_pair<P>(x.sts, p, ty);
+      acc_batch(acc, x.sts, p, ty);
     }
   }
+  acc_end(acc, x.sts);
 }
 
 // UpperBound of the round-0 items: every face of every pair (tri == nullptr), or n given
@@ -527,6 +596,8 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
                          });
     return;
   }
+  __shared__ PairAcc s_acc[kMaxWarps];
+  PairAcc& acc = acc_begin(s_acc);
   for (;;) {
     const int base = warp_batch(&bs->b_next);
     if (base >= count) break;
@@ -555,17 +626,16 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
         }
       }
     }
-    Counters cnt;
-    PairTally<P> ty;
+    PairDelta<P> ty;
     if (p >= 0) {
       const PairLevel<P> pl = pair_level<P>(x, p);
       int code;
-      it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, cnt);
+      it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, ty.c);
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    flush_counters_pair(x.sts, p, cnt);
-    flush_tally_pair<P>(x.sts, p, ty);
+    acc_batch(acc, x.sts, p, ty);
   }
+  acc_end(acc, x.sts);
 }
 
 // The pass over the items the UpperBound kernel left (bound_u4_body), with full warps.
@@ -578,25 +648,26 @@ __global__ void k_batch_bound_u4(BatchCtx x, const typename P::Vtx* pool, const 
   BatchState* bs = x.bs;
   if (round_midpoints && bs->stop) return;
   const int n = min(*(volatile int*)&bs->n_u4, cap);
+  __shared__ PairAcc s_acc[kMaxWarps];
+  PairAcc& acc = acc_begin(s_acc);
   // warp-uniform loop: each warp takes 32 consecutive items per step
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n;
        base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = base + (threadIdx.x & 31);
     int p = -1;
-    Counters cnt;
-    PairTally<P> ty;
+    PairDelta<P> ty;
     if (t < n) {
       p = u4_pair[t];
       typename P::Item it = u4list[t];
       const PairLevel<P> pl = pair_level<P>(x, p);
       int code;
       P::bound_deferred(x.pd[p].B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.lv.l, pl.lv.th.lo, pl.rp, it.U, code,
-                        cnt);
+                        ty.c);
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, nullptr, nullptr, ty);
     }
-    if constexpr (P::kFp64) flush_counters_pair(x.sts, p, cnt);
-    flush_tally_pair<P>(x.sts, p, ty);
+    acc_batch(acc, x.sts, p, ty);
   }
+  acc_end(acc, x.sts);
 }
 
 // Select (Section 3.1 / 4): every item of a running pair with U > l + eps is split while the
@@ -614,12 +685,14 @@ __global__ void k_batch_select(BatchCtx x, const typename P::Item* front, const 
   BatchState* bs = x.bs;
   if (bs->stop) return;
   const int n_front = bs->n_front, K = bs->K, mbase = bs->n_pool;
+  __shared__ PairAcc s_acc[kMaxWarps];
+  PairAcc& acc = acc_begin(s_acc);
   // warp-uniform loop: each warp takes 32 consecutive items per step
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n_front;
        base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = base + (threadIdx.x & 31);
     int p = -1;
-    PairTally<P> ty;
+    PairDelta<P> ty;
     if (i < n_front) {
       p = front_pair[i];
       if (x.sts[p].stop) p = -1;  // the pair is done: its items go
@@ -650,8 +723,13 @@ __global__ void k_batch_select(BatchCtx x, const typename P::Item* front, const 
         } else {
           const int s = warp_slot(&bs->n_split);
           if (s < K) {
-            // the pair's face cap: splits of earlier rounds plus this round's so far
-            const int k = atomicAdd(&x.sts[p].n_split, 1);
+            // the pair's face cap: splits of earlier rounds plus this round's so far (one
+            // atomic per pair of the warp)
+            namespace cg = cooperative_groups;
+            const auto g = cg::labeled_partition(cg::coalesced_threads(), p);
+            int k = 0;
+            if (g.thread_rank() == 0) k = atomicAdd(&x.sts[p].n_split, (int)g.size());
+            k = g.shfl(k, 0) + (int)g.thread_rank();
             const bool ok = x.sts[p].splits + k < x.pd[p].splits_cap;
             if (!ok) {
               atomicSub(&x.sts[p].n_split, 1);
@@ -690,8 +768,9 @@ __global__ void k_batch_select(BatchCtx x, const typename P::Item* front, const 
         }
       }
     }
-    flush_tally_pair<P>(x.sts, p, ty);
+    acc_batch(acc, x.sts, p, ty);
   }
+  acc_end(acc, x.sts);
 }
 
 // The four children of every split (Section 4, midpoint subdivision), bounded with their
@@ -725,6 +804,8 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
                          });
     return;
   }
+  __shared__ PairAcc s_acc[kMaxWarps];
+  PairAcc& acc = acc_begin(s_acc);
   for (;;) {
     const int64_t base = warp_batch(&bs->b_next);
     if (base >= 4 * (int64_t)S) break;
@@ -736,8 +817,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
       k = (int)(t & 3);
       p = split_pair[s];
     }
-    Counters cnt;
-    PairTally<P> ty;
+    PairDelta<P> ty;
     if (p >= 0) {
       const int4 par = split_par[s];
       const int m12 = mbase + 3 * s, m23 = m12 + 1, m31 = m12 + 2;
@@ -748,15 +828,15 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
       else { it.v[0] = m12; it.v[1] = m23; it.v[2] = m31; }
       const PairLevel<P> pl = pair_level<P>(x, p);
       int code;
-      it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, cnt);
+      it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, ty.c);
       // the child lies inside its parent: h(child, B) <= U(parent)
       const typename P::UT Up = (typename P::UT)__int_as_float(par.w);
       if (pl.rp.parent_clamp && Up < it.U) it.U = Up;
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    flush_counters_pair(x.sts, p, cnt);
-    flush_tally_pair<P>(x.sts, p, ty);
+    acc_batch(acc, x.sts, p, ty);
   }
+  acc_end(acc, x.sts);
 }
 
 // The UpperBound kernels of policy P: the straight-line paper-order instantiation or the

@@ -408,28 +408,33 @@ __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned
     b1 = along(v1, e12, s2, be1);
     b2 = along(v1, e13, s3, be2);
   }
-  float d[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    // case 2 slot k: triangle of vertex k / 2, and the next or the other vertex
-    const int i = k >> 1, j = (k == 0 || k == 5) ? 1 : ((k == 1 || k == 3) ? 2 : 0);
-    FFP x = c1 ? ((k & 1) ? b2 : b1) : t[j].p;
-    float be = c1 ? ((k & 1) ? be2 : be1) : 0.f;
-    int S = c1 ? (k < 2 ? S1 : S2) : t[i].I;
-    d[k] = (c1 && k >= 4) ? 0.f : dist_hi(B, S, x, be);
-  }
   const float dmax = fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi));
+  // The slots, two at a time.  The loops below are not unrolled: with every evaluation inlined
+  // (15 copies of the point-triangle code) the kernels outgrew the instruction cache, and
+  // waiting for instructions was their largest stall (4 to 6 cycles per instruction issued,
+  // now 1 to 1.7).  On the batch of 128 pairs the bounds went from 21.7 to 18.6 ms, on the
+  // large soup from 0.093 to 0.083 ms; the torus pair's stayed at 0.10 ms.  The loops keep
+  // their points in local memory, so they want 128 registers (96: 18.6, 0.089, 0.109 ms).
+  float u = dmax, best = INFINITY;
+#pragma unroll 1
+  for (int i = 0; i < (c1 ? 2 : 3); ++i) {
+    // case 1: both split points against S1, then S2; case 2: the two other vertices against S_i
+    const VM &x = i == 0 ? t[1] : i == 1 ? t[2] : t[0], &y = i == 0 ? t[2] : i == 1 ? t[0] : t[1];
+    const int S = c1 ? (i == 0 ? S1 : S2) : i == 0 ? t[0].I : i == 1 ? t[1].I : t[2].I;
+    const float own = i == 0 ? t[0].dhi : i == 1 ? t[1].dhi : t[2].dhi;
+    const FFP p0 = c1 ? b1 : x.p, p1 = c1 ? b2 : y.p;
+    const float d = fmaxf(dist_hi(B, S, p0, c1 ? be1 : 0.f), dist_hi(B, S, p1, c1 ? be2 : 0.f));
+    u = fmaxf(u, d);
+    best = fminf(best, fmaxf(own, d));
+  }
   if (c1) {
     evals += 4;
-    const float u = fmaxf(dmax, fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])));
     return kAgree ? __fadd_ru(u, apart) : u;
   }
   // case 2: u3 = min(u3~, min_i h(T, S_i)).  The second term comes from the slots: once it is
   // below l the item is discarded whatever u3~ is (U of a discarded item is not used
   // further), and the quadrilateral maximum u3~ is abandoned as soon as it reaches the
   // current minimum, since it can then no longer lower it.
-  float best = fminf(fmaxf(t[0].dhi, fmaxf(d[0], d[1])),
-                     fminf(fmaxf(t[1].dhi, fmaxf(d[2], d[3])), fmaxf(t[2].dhi, fmaxf(d[4], d[5]))));
   evals += 6;
   if (best < l) return best;
   // quadrilaterals (v_i, m_i, b, m_{i-1}) against S_i
@@ -444,14 +449,17 @@ __device__ inline float ubm_u3(const BvhDev& B, const VM t[3], float l, unsigned
   FFP bc = along(t[0], sum, 1.f / 3.f, bb);
   bb = __fmul_ru(16.f * kU, fmaxf(amax3(e01), fmaxf(amax3(e02), amax3(t[0].p.l))));
   float ut = dmax;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (ut >= best) break;
-    int S = t[i].I;
-    ut = fmaxf(ut, dist_hi(B, S, m[i], bm[i]));
-    ut = fmaxf(ut, dist_hi(B, S, bc, bb));
-    ut = fmaxf(ut, dist_hi(B, S, m[(i + 2) % 3], bm[(i + 2) % 3]));
-    evals += 3;
+#pragma unroll 1
+  for (int k = 0; k < 9; ++k) {
+    const int i = k / 3, j = k - 3 * i;  // j: m_i, b, m_{i-1}
+    if (j == 0) {
+      if (ut >= best) break;
+      evals += 3;
+    }
+    const int S = i == 0 ? t[0].I : i == 1 ? t[1].I : t[2].I;
+    const int q = j == 0 ? i : i == 0 ? 2 : i - 1;
+    const FFP x = j == 1 ? bc : q == 0 ? m[0] : q == 1 ? m[1] : m[2];
+    ut = fmaxf(ut, dist_hi(B, S, x, j == 1 ? bb : q == 0 ? bm[0] : q == 1 ? bm[1] : bm[2]));
   }
   return fminf(ut, best);
 }

@@ -539,7 +539,7 @@ __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const dou
 #define HD_FP64_BOUND_REGS 128
 #endif
 #ifndef HD_FP64_PAPER_REGS
-#define HD_FP64_PAPER_REGS 96
+#define HD_FP64_PAPER_REGS 128
 #endif
 
 struct PolicyD {

@@ -493,7 +493,7 @@ __device__ inline float upper_bound_m_paper(const BvhDev& B, const VM t[3], floa
 #define HD_MIXED_BOUND_REGS 96
 #endif
 #ifndef HD_MIXED_PAPER_REGS
-#define HD_MIXED_PAPER_REGS 96
+#define HD_MIXED_PAPER_REGS 128
 #endif
 
 struct PolicyM {
