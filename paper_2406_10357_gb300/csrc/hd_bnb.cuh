@@ -57,13 +57,34 @@ __device__ inline double warp_max(double v) {
   return v;
 }
 
-// The next batch of 32 consecutive items for the calling warp (every lane must call it):
+// The next batch of `take` consecutive items for the calling warp (every lane must call it):
 // warps of a persistent grid take batches until `count` is reached, so the grid's last
 // wave is not left to a few blocks.
-__device__ inline int warp_batch(int* counter) {
+__device__ inline int warp_batch(int* counter, int take = 32) {
   int base = 0;
-  if ((threadIdx.x & 31) == 0) base = atomicAdd(counter, 32);
+  if ((threadIdx.x & 31) == 0) base = atomicAdd(counter, take);
   return __shfl_sync(0xffffffffu, base, 0);
+}
+
+// Items a warp takes at a time (a power of two, at most 32) from a list of `count`: fewer than
+// 32 where the list is too short to give every warp that many.  A short list is bound by the
+// time of its slowest warp, and a warp takes the longer the more lanes diverge in it; spread
+// over more warps, each waits for fewer others.  `per_sm` is the warps per SM worth filling
+// that way.  The FP64 pipe takes as long for one lane as for 32, so FP64 bounds want few.
+// The two 320-triangle spheres in FP64: 1190 -> 836 us per pair; 1000 points, MIXED: 80 -> 49 us
+// (2, 4, 8, 16 warps per SM: 57, 54, 49, 49).  FP64 queries of the two-sided scan with 1, 2, 4,
+// 8: 0.93, 0.87, 0.80, 0.76 ms; its bounds 0.79, 0.78, 0.81, 0.97 ms.
+constexpr int kSms = 152;
+__device__ inline int spread_lanes(int64_t count, int per_sm) {
+  const int64_t warps = min((int64_t)gridDim.x * (blockDim.x >> 5), (int64_t)per_sm * kSms);
+  int lanes = 32;
+  while (lanes > 1 && count <= (lanes >> 1) * warps) lanes >>= 1;
+  return lanes;
+}
+// Blocks of bs threads for a list of at most n items spread that way, at most `most`.
+inline unsigned spread_grid(int64_t n, int bs, unsigned most, int per_sm) {
+  const int64_t w = std::min<int64_t>(std::max<int64_t>(n, 1), (int64_t)per_sm * kSms);
+  return std::min(std::max(blocks_for(n, bs), blocks_for(32 * w, bs)), most);
 }
 
 // Flush per-thread counters with one atomic per warp.  Every lane of the warp must call it.
@@ -314,7 +335,7 @@ __device__ inline unsigned long_bucket(const BvhDev& B, float px, float py, floa
 
 // Nearest-triangle queries for pool vertices [beg, beg + count); count = min(*count_ptr *
 // mult, cap) when count_ptr is given (device-side counts), else `cap`.  Warps take batches of
-// 32 consecutive vertices, one per lane, each lane traversing on its own (the while-while
+// 32 consecutive vertices (fewer of a short list: spread_lanes), one per lane, each lane traversing on its own (the while-while
 // traversal).  With a list, a lane whose traversal tests more than kLongBudget triangles
 // stops and hands its query to k_query_long, which runs next and counts it.  Registers are
 // capped at 128 (a few spilled to L1), for 8 resident blocks of 64 threads per SM.
@@ -338,21 +359,22 @@ __device__ inline void query_body(BvhDev B, typename P::Vtx* pool, int beg, cons
   }
   const double slack = dyn ? dyn->slack : slack_in;
   const bool cutting = HD_CUT_LANE && cut_on(dyn);
-  // With cuts, the batches of 32 are taken from kQuerySegments interleaved parts of the
+  // With cuts, the batches are taken from kQuerySegments interleaved parts of the
   // list, so that vertices from every part of A (the far ones among them) raise l early and
   // the queries after them cut sooner; each part is still taken in order.
-  const int nb = (count + 31) >> 5, segs = cutting ? kQuerySegments : 1, per = (nb + segs - 1) / segs;
+  const int lanes = spread_lanes(count, P::kSpread), sh = 31 - __clz(lanes);
+  const int nb = (count + lanes - 1) >> sh, segs = cutting ? kQuerySegments : 1, per = (nb + segs - 1) / segs;
   Counters c;
   double lmax = 0.0;
   int nq = 0, ncut = 0;
   for (;;) {
-    const int b = warp_batch(&st->q_next) >> 5;
+    const int b = warp_batch(&st->q_next, lanes) >> sh;
     if (b >= segs * per) break;
-    const int base = ((b % segs) * per + b / segs) << 5;
+    const int base = ((b % segs) * per + b / segs) << sh;
     if (base >= count) continue;
     const double lnow = cutting ? read_lower(st) : 0.0;
     const int t = base + (threadIdx.x & 31);
-    bool active = t < count;
+    bool active = (threadIdx.x & 31) < lanes && t < count;
     // every lane of the warp enters the query (the MIXED traversal votes across the warp);
     // lanes without a vertex to query take part as already finished
     typename P::Vtx v;
@@ -415,7 +437,7 @@ __global__ void HD_QUERY_REGS k_query(BvhDev B, typename P::Vtx* pool, int beg, 
 // The queries k_query handed off, one warp each (traverse_coop, with this warp's stack in
 // shared memory), taken one at a time from a counter since their costs vary widely; with
 // their contribution to l and to the query counts.
-template <class P>
+template <class P, bool kCuts>
 __device__ inline void query_long_body(BvhDev B, typename P::Vtx* pool, LongList ll, RunState* st, double slack_in,
                                        const DynParams* dyn, bool round_midpoints, unsigned* s_code, float* s_e) {
   if (round_midpoints && st->stop) return;  // as k_query (uniform over the grid)
@@ -428,7 +450,7 @@ __device__ inline void query_long_body(BvhDev B, typename P::Vtx* pool, LongList
   const int* list = sorted ? ll.sorted : ll.idx;
   // (ordered by cost with cuts: one at a time, so that the costly ones spread over the warps)
   const int chunk = sorted && !(HD_LONG_LPT && cut_on(dyn)) ? kLongChunk : 1;
-  const bool cutting = HD_CUT_LONG && cut_on(dyn);
+  const bool cutting = kCuts && HD_CUT_LONG && cut_on(dyn);
   Counters c;
   double lmax = 0.0;
   int nq = 0, ncut = 0;
@@ -463,15 +485,18 @@ __device__ inline void query_long_body(BvhDev B, typename P::Vtx* pool, LongList
   flush_counters(st, c, true);
 }
 
-template <class P>
-__global__ void __launch_bounds__(32 * kCoopWarps, P::kCoopBlocks) k_query_long(BvhDev B, typename P::Vtx* pool, LongList ll,
-                                                                RunState* st, double slack_in, const DynParams* dyn,
-                                                                bool round_midpoints) {
+// With kCuts the queries may be cut (the host's cut_enabled); a kernel that never cuts holds
+// one traversal instead of two and fits more blocks per SM (500,000 points near a torus,
+// MIXED, 0.661 -> 0.617 ms per call).
+template <class P, bool kCuts>
+__global__ void __launch_bounds__(32 * kCoopWarps, kCuts ? P::kCoopBlocksCut : P::kCoopBlocks)
+    k_query_long(BvhDev B, typename P::Vtx* pool, LongList ll, RunState* st, double slack_in, const DynParams* dyn,
+                 bool round_midpoints) {
   __shared__ unsigned s_code[kCoopWarps * kCoopStack];
   __shared__ float s_e[kCoopWarps * kCoopStack];
   grid_dep_wait();
   grid_dep_launch();
-  query_long_body<P>(B, pool, ll, st, slack_in, dyn, round_midpoints, s_code, s_e);
+  query_long_body<P, kCuts>(B, pool, ll, st, slack_in, dyn, round_midpoints, s_code, s_e);
 }
 
 // The reordering of a long-query list along the Morton curve of its points (a counting sort on
@@ -515,17 +540,13 @@ __global__ void k_long_hist(BvhDev B, const typename P::Vtx* pool, LongList ll, 
 
 // Exclusive scan of the cell counts: one block of 1024 threads, kSortBuckets / 1024 rows of
 // 1024 consecutive counters, each row scanned across the block (coalesced) and carried on.
-static __global__ void k_long_scan(LongList ll, const RunState* st, bool round_midpoints) {
-  grid_dep_wait();
-  grid_dep_launch();
-  if (round_midpoints && st->stop) return;
-  if (min(st->n_long, ll.cap) < kSortMin) return;
+__device__ inline void scan_buckets(unsigned* buckets) {
   constexpr int kRows = kSortBuckets / 1024;
   __shared__ unsigned wtot[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   unsigned val[kRows];  // every row's counter first: the loads overlap instead of one per row
 #pragma unroll
-  for (int row = 0; row < kRows; ++row) val[row] = ll.buckets[row * 1024 + threadIdx.x];
+  for (int row = 0; row < kRows; ++row) val[row] = buckets[row * 1024 + threadIdx.x];
   unsigned carry = 0;
 #pragma unroll
   for (int row = 0; row < kRows; ++row) {
@@ -547,10 +568,18 @@ static __global__ void k_long_scan(LongList ll, const RunState* st, bool round_m
       wtot[lane] = t;
     }
     __syncthreads();
-    ll.buckets[i] = carry + (w ? wtot[w - 1] : 0u) + x - v;
+    buckets[i] = carry + (w ? wtot[w - 1] : 0u) + x - v;
     carry += wtot[31];
     __syncthreads();  // wtot is written again by the next row
   }
+}
+
+static __global__ void k_long_scan(LongList ll, const RunState* st, bool round_midpoints) {
+  grid_dep_wait();
+  grid_dep_launch();
+  if (round_midpoints && st->stop) return;
+  if (min(st->n_long, ll.cap) < kSortMin) return;
+  scan_buckets(ll.buckets);
 }
 
 template <class P>
@@ -807,11 +836,12 @@ __global__ void HD_BOUND_REGS k_bound_faces(BvhDev B, const typename P::Vtx* poo
     flush_tally(st, ty);
     return;
   }
+  const int lanes = spread_lanes(nFA, P::kSpreadBounds);
   for (;;) {
-    const int64_t base = warp_batch(&st->b_next);
+    const int64_t base = warp_batch(&st->b_next, lanes);
     if (base >= nFA) break;
     const int64_t f = base + (threadIdx.x & 31);
-    if (f >= nFA) continue;
+    if ((threadIdx.x & 31) >= lanes || f >= nFA) continue;
     typename P::Item it;
     it.v[0] = FA[3 * f];
     it.v[1] = FA[3 * f + 1];
@@ -841,7 +871,11 @@ __device__ inline void bound_u4_body(BvhDev B, const typename P::Vtx* pool, cons
   const Thresholds<P>& th = lv.th;
   Counters c;
   Tally<P> ty;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+  const int lanes = spread_lanes(n, P::kSpreadBounds), lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  for (int64_t base = (blockIdx.x * (int64_t)wpb + (threadIdx.x >> 5)) * lanes; base < n;
+       base += (int64_t)gridDim.x * wpb * lanes) {
+    const int64_t t = base + lane;
+    if (lane >= lanes || t >= n) continue;
     typename P::Item it = u4list[t];
     int code;
     P::bound_deferred(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.l, th.lo, rp, it.U, code, c);
@@ -1040,11 +1074,12 @@ __device__ inline void bound_children_body(BvhDev B, const typename P::Vtx* pool
     flush_tally(st, ty);
     return;
   }
+  const int lanes = spread_lanes(4 * (int64_t)S, P::kSpreadBounds);
   for (;;) {
-    const int64_t base = warp_batch(&st->b_next);
+    const int64_t base = warp_batch(&st->b_next, lanes);
     if (base >= 4 * (int64_t)S) break;
     const int64_t t = base + (threadIdx.x & 31);
-    if (t < 4 * (int64_t)S) {
+    if ((threadIdx.x & 31) < lanes && t < 4 * (int64_t)S) {
       int s = (int)(t >> 2), k = (int)(t & 3);
       const int4 par = split_par[s];
       const int4 mid = share ? split_mid[s] : make_int4(mbase + 3 * s, mbase + 3 * s + 1, mbase + 3 * s + 2, 0);
@@ -1261,7 +1296,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_rounds(BvhDev B, TailBufs
     __syncthreads();
     query_body<P>(B, a.pool, 0, nullptr, 3, 0, st, rp.slack, rp.dyn, true, a.tab, lq);
     __syncthreads();
-    query_long_body<P>(B, a.pool, lq, st, rp.slack, rp.dyn, true, s_code, s_e);
+    query_long_body<P, true>(B, a.pool, lq, st, rp.slack, rp.dyn, true, s_code, s_e);
     __syncthreads();
     typename P::Item* left = a.u4list ? a.u4list : a.front[cur];
     bound_children_body<P>(B, a.pool, a.split_par, a.split_mid, st, rp, a.front[cur ^ 1], a.front_cap, left);
@@ -1432,10 +1467,22 @@ unsigned query_grid(int bs) {
   static std::atomic<unsigned> cache[33];
   return persistent_grid_bs(k_query<P>, bs, cache);
 }
-template <class P>
+template <class P, bool kCuts>
 unsigned long_grid() {
   static std::atomic<unsigned> cache[33];
-  return persistent_grid_bs(k_query_long<P>, 32 * kCoopWarps, cache);
+  return persistent_grid_bs(k_query_long<P, kCuts>, 32 * kCoopWarps, cache);
+}
+
+// k_query_long over the handed-off queries of the k_query launch before it.
+template <class P>
+void launch_query_long(bool cuts, const BvhDev& B, typename P::Vtx* pool, const LongList& ll, RunState* st, double slack,
+                       const DynParams* dyn, bool round_midpoints, cudaStream_t s) {
+  if (cuts)
+    launch_chained(k_query_long<P, true>, long_grid<P, true>(), 32 * kCoopWarps, 0, s, B, pool, ll, st, slack, dyn,
+                   round_midpoints);
+  else
+    launch_chained(k_query_long<P, false>, long_grid<P, false>(), 32 * kCoopWarps, 0, s, B, pool, ll, st, slack, dyn,
+                   round_midpoints);
 }
 
 struct Totals {
@@ -1599,7 +1646,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
   const size_t smem_b = rebin_smem(bs);  // the u3 queues of the paper-order kernels
   const unsigned grid_q = query_grid<P>(bs),
                  grid_b = persistent_grid_bs(k_children, bs, grid_b_cache[paper ? 1 : 0], smem_b);
-  const unsigned grid_long = long_grid<P>();
+  const bool cuts = cut_enabled(o);
   int64_t front_bound = first_front_bound;  // the first round is queued without a wait
   int cur = R.cur;
   bool init = true;
@@ -1615,8 +1662,8 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     // grids for a frontier of at most nf items (grid-stride kernels: any size is correct)
     const int64_t k = std::max<int64_t>(1, std::min<int64_t>(nf, R.chunk));
     const unsigned g_sel = std::min(blocks_for(std::max<int64_t>(nf, 1), 256), (unsigned)sms * 8);
-    const unsigned g_q = std::min(blocks_for(3 * k, bs), grid_q), g_b = std::min(blocks_for(4 * k, bs), grid_b);
-    const unsigned g_u4 = std::min(blocks_for(4 * k, bs), max_grid);
+    const unsigned g_q = spread_grid(3 * k, bs, grid_q, P::kSpread), g_b = spread_grid(4 * k, bs, grid_b, P::kSpreadBounds);
+    const unsigned g_u4 = spread_grid(4 * k, pass_block<P>(bs), max_grid, P::kSpreadBounds);
     {
       TraceScope tr(HD_K_SELECT, s);
       launch_chained(k_round_ctl, 1, 1, 0, s, st, c, init ? 1 : 0, n_pool0);
@@ -1632,7 +1679,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     {
       TraceScope tr(HD_K_LONG, s);
       sort_long<P>(B, R.pool, R.longq, st, true, sms, s, rp.dyn);
-      launch_chained(k_query_long<P>, grid_long, 32 * kCoopWarps, 0, s, B, R.pool, R.longq, st, rp.slack, rp.dyn, true);
+      launch_query_long<P>(cuts, B, R.pool, R.longq, st, rp.slack, rp.dyn, true, s);
     }
     {
       TraceScope tr(HD_K_BOUND, s);
@@ -1786,7 +1833,8 @@ int finish_in_fp64(const RunIO& io, Rounds<P>& RM, int64_t n_pro, RunState* st, 
   HD_TRY_LAUNCH();
   {
     TraceScope tr(HD_K_QUERY, s);
-    launch_chained(k_query<PolicyD>, blocks_for(3 * n_pro, o.block_size), o.block_size, 0, s,
+    launch_chained(k_query<PolicyD>, spread_grid(3 * n_pro, o.block_size, query_grid<PolicyD>(o.block_size), PolicyD::kSpread),
+                   o.block_size, 0, s,
         B, D.pool, 0, nullptr, 1, (int)(3 * n_pro), st, rp.slack, rp.dyn, false, MidTable{nullptr, nullptr, nullptr, 0},
         D.longq);
   }
@@ -1796,15 +1844,14 @@ int finish_in_fp64(const RunIO& io, Rounds<P>& RM, int64_t n_pro, RunState* st, 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sort_long<PolicyD>(B, D.pool, D.longq, st, false, sms, s, rp.dyn);
-    launch_chained(k_query_long<PolicyD>, long_grid<PolicyD>(), 32 * kCoopWarps, 0, s, B, D.pool, D.longq, st, rp.slack,
-                   rp.dyn, false);
+    launch_query_long<PolicyD>(cut_enabled(o), B, D.pool, D.longq, st, rp.slack, rp.dyn, false, s);
   }
   {
     TraceScope tr(HD_K_BOUND, s);
     const auto k_faces = bound_faces_kernel<PolicyD>(paper_cascade(rp));
-    launch_chained(k_faces, blocks_for(n_pro, o.block_size), o.block_size, rebin_smem(o.block_size), s, B, D.pool, tris,
+    launch_chained(k_faces, spread_grid(n_pro, o.block_size, 65535u, PolicyD::kSpreadBounds), o.block_size, rebin_smem(o.block_size), s, B, D.pool, tris,
                    n_pro, st, rp, D.front[1], (int)D.front_cap, D.left(1), 3 * n_pro);
-    launch_chained(k_bound_u4<PolicyD>, blocks_for(n_pro, pass_block<PolicyD>(o.block_size)),
+    launch_chained(k_bound_u4<PolicyD>, spread_grid(n_pro, pass_block<PolicyD>(o.block_size), 65535u, PolicyD::kSpreadBounds),
                    pass_block<PolicyD>(o.block_size), 0, s, B, D.pool, (const ItemD*)D.left(1), (int)D.front_cap, st, rp,
                    D.front[1], (int)D.front_cap);
   }
@@ -1882,20 +1929,20 @@ int run_bnb(const RunIO& io) {
   // round 0: vertices of A, their nearest triangles, l, and the bounds of every face
   {
     TraceScope tr(HD_K_QUERY, s);
-    launch_chained(k_query<P>, std::min(blocks_for(io.nVA, bs), query_grid<P>(bs)), bs, 0, s,
+    launch_chained(k_query<P>, spread_grid(io.nVA, bs, query_grid<P>(bs), P::kSpread), bs, 0, s,
         B, R.pool, 0, nullptr, 1, (int)io.nVA, st, rp.slack, rp.dyn, false, MidTable{nullptr, nullptr, nullptr, 0},
         R.longq);
   }
   {
     TraceScope tr(HD_K_LONG, s);
     sort_long<P>(B, R.pool, R.longq, st, false, sms, s, rp.dyn);
-    launch_chained(k_query_long<P>, long_grid<P>(), 32 * kCoopWarps, 0, s, B, R.pool, R.longq, st, rp.slack, rp.dyn, false);
+    launch_query_long<P>(cut_enabled(o), B, R.pool, R.longq, st, rp.slack, rp.dyn, false, s);
   }
   HD_TRY_LAUNCH();
   {
     TraceScope tr(HD_K_BOUND, s);
     const auto k_faces = bound_faces_kernel<P>(paper_cascade(rp));
-    launch_chained(k_faces, std::min(blocks_for(io.nFA, bs), persistent_grid(k_faces, bs, sms, rebin_smem(bs))), bs,
+    launch_chained(k_faces, spread_grid(io.nFA, bs, persistent_grid(k_faces, bs, sms, rebin_smem(bs)), P::kSpreadBounds), bs,
                    rebin_smem(bs), s, 
         B, R.pool, io.FA, io.nFA, st, rp, R.front[1],
                                                            (int)R.front_cap, R.left(1), io.nVA);
@@ -1964,8 +2011,60 @@ int run_bnb(const RunIO& io) {
 
 // ----------------------------------------------------------------------------- point queries
 
+// The order external points are queried in.  Points that follow each other in space share
+// nodes and branches in a warp; points in random order share neither.  So a large set is
+// grouped by Morton cell of B's box (a counting sort: k_points_cell, k_points_scan,
+// k_points_place), unless its own order is coherent already, that is, unless few neighbours
+// lie in different cells; the results go back in the caller's order, and each query's result
+// does not depend on its place.  500,000 random points near a torus of 50,176 triangles,
+// MIXED: 0.724 -> 0.661 ms per call, the sort included.  Below kPointSortMin points the
+// queries are bound by their latency and the sort does not pay.
+struct PointOrder {
+  int* place = nullptr;  // record of each point (null: the points' own order)
+  int* cell = nullptr;
+  unsigned* buckets = nullptr;  // kSortBuckets counters, zero at the start
+  unsigned* jumps = nullptr;    // neighbouring points in different cells, zero at the start
+};
+constexpr int64_t kPointSortMin = 1 << 15;
+
+__device__ inline bool points_sorted(const PointOrder& o, int64_t n) {
+  return o.place && (int64_t)*o.jumps * 4 > n;
+}
+
+template <typename T>
+__global__ void k_points_cell(BvhDev B, const T* P_, int64_t n, PointOrder o) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const bool on = i < n;
+  const int c = on ? (int)long_bucket(B, (float)P_[3 * i], (float)P_[3 * i + 1], (float)P_[3 * i + 2]) : -1;
+  const int before = __shfl_up_sync(0xffffffffu, c, 1);
+  const unsigned j = __ballot_sync(0xffffffffu, on && lane > 0 && c != before);
+  const unsigned same = __match_any_sync(0xffffffffu, c);
+  if (on) {
+    o.cell[i] = c;
+    if (lane == __ffs(same) - 1) atomicAdd(&o.buckets[c], (unsigned)__popc(same));
+  }
+  if (lane == 0 && j) atomicAdd(o.jumps, (unsigned)__popc(j));
+}
+
+static __global__ void k_points_scan(PointOrder o, int64_t n) {
+  grid_dep_wait();
+  grid_dep_launch();
+  if (points_sorted(o, n)) scan_buckets(o.buckets);
+}
+
+static __global__ void k_points_place(PointOrder o, int64_t n) {
+  grid_dep_wait();
+  grid_dep_launch();
+  if (!points_sorted(o, n)) return;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) o.place[i] = (int)atomicAdd(&o.buckets[o.cell[i]], 1u);
+}
+
 template <class P, typename T>
-__global__ void k_points_in(const T* P_, int64_t n, typename P::Vtx* v) {
+__global__ void k_points_in(const T* P_, int64_t n, typename P::Vtx* v, PointOrder o) {
   grid_dep_wait();
   grid_dep_launch();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1975,17 +2074,17 @@ __global__ void k_points_in(const T* P_, int64_t n, typename P::Vtx* v) {
   P::set_pos(x, (double)P_[3 * i], (double)P_[3 * i + 1], (double)P_[3 * i + 2]);
   x.tri = -2;
   x.hint = -1;
-  v[i] = x;
+  v[points_sorted(o, n) ? o.place[i] : i] = x;
 }
 
 template <class P>
 __global__ void k_points_out(const typename P::Vtx* v, int64_t n, const int4* tri_vid, double* dist, int32_t* idx,
-                             double* foot, double* dlo) {
+                             double* foot, double* dlo, PointOrder o) {
   grid_dep_wait();
   grid_dep_launch();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  typename P::Vtx x = v[i];
+  typename P::Vtx x = v[points_sorted(o, n) ? o.place[i] : i];
   dist[i] = P::out_dist(x);
   idx[i] = x.tri >= 0 ? tri_vid[x.tri].w : -1;
   D3 f = P::out_foot(x);
@@ -2003,7 +2102,7 @@ void query_points(const BvhDev& B, typename P::Vtx* rec, int64_t n, RunState* st
                   int* sorted = nullptr, unsigned* buckets = nullptr) {
   if (list && n <= INT32_MAX / 2) {
     const LongList ll = {list, (int)n, sorted, buckets};
-    launch_chained(k_query<P>, std::min(blocks_for(n, 128), query_grid<P>(128)), 128, 0, s, B, rec, 0, nullptr, 1,
+    launch_chained(k_query<P>, spread_grid(n, 128, query_grid<P>(128), P::kSpread), 128, 0, s, B, rec, 0, nullptr, 1,
                    (int)n, st, 0.0, nullptr, false, MidTable{nullptr, nullptr, nullptr, 0}, ll);
     if (sorted) {
       int dev = 0, sms = 1;
@@ -2011,7 +2110,7 @@ void query_points(const BvhDev& B, typename P::Vtx* rec, int64_t n, RunState* st
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       sort_long<P>(B, rec, ll, st, false, sms, s, nullptr);
     }
-    launch_chained(k_query_long<P>, long_grid<P>(), 32 * kCoopWarps, 0, s, B, rec, ll, st, 0.0, nullptr, false);
+    launch_query_long<P>(false, B, rec, ll, st, 0.0, nullptr, false, s);
   } else {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -2024,35 +2123,54 @@ void query_points(const BvhDev& B, typename P::Vtx* rec, int64_t n, RunState* st
 template <class P>
 int nearest_points(const hd_bvh* B, const void* Pts, int ptype, int64_t n, cudaStream_t s, double* dist,
                    int32_t* idx, double* foot, double* dlo) {
-  typename P::Vtx* tmp = nullptr;
-  RunState* st = nullptr;
-  int* list = nullptr;
-  int* sorted = nullptr;
-  unsigned* buckets = nullptr;
   const bool two_phase = n <= INT32_MAX / 2;  // k_query counts in int
-  HD_TRY(cudaMallocAsync((void**)&tmp, sizeof(typename P::Vtx) * n, s));
-  HD_TRY(cudaMallocAsync((void**)&st, sizeof(RunState), s));
-  if (two_phase) HD_TRY(cudaMallocAsync((void**)&list, sizeof(int) * n, s));
-  if (two_phase && n >= kSortMin) {
-    HD_TRY(cudaMallocAsync((void**)&sorted, sizeof(int) * n, s));
-    HD_TRY(cudaMallocAsync((void**)&buckets, sizeof(unsigned) * kSortBuckets, s));
+  const bool sort_list = two_phase && n >= kSortMin, sort_in = two_phase && n >= kPointSortMin;
+  // one allocation: the records, the lists of the two phases, the points' places, and what
+  // starts at zero (run state, jumps, cell counters) at the end
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t b_rec = up(sizeof(typename P::Vtx) * n), b_list = two_phase ? up(sizeof(int) * n) : 0,
+               b_sorted = sort_list ? b_list : 0, b_place = sort_in ? b_list : 0, b_st = up(sizeof(RunState) + 4),
+               b_buckets = sort_list ? sizeof(unsigned) * kSortBuckets : 0;
+  char* base = nullptr;
+  HD_TRY(cudaMallocAsync((void**)&base, b_rec + b_list + b_sorted + b_place + b_st + b_buckets, s));
+  typename P::Vtx* tmp = (typename P::Vtx*)base;
+  int* list = two_phase ? (int*)(base + b_rec) : nullptr;
+  int* sorted = sort_list ? (int*)(base + b_rec + b_list) : nullptr;
+  char* zero = base + b_rec + b_list + b_sorted + b_place;
+  RunState* st = (RunState*)zero;
+  unsigned* buckets = sort_list ? (unsigned*)(zero + b_st) : nullptr;
+  cudaError_t e = cudaMemsetAsync(zero, 0, b_st + (sort_in ? b_buckets : 0), s);
+  if (e != cudaSuccess) {
+    cudaFreeAsync(base, s);
+    return set_cuda_error(e, "cudaMemsetAsync", __FILE__, __LINE__);
   }
-  HD_TRY(cudaMemsetAsync(st, 0, sizeof(RunState), s));
+  PointOrder o;
+  if (sort_in) {  // the cells stay in the list's room until the queries start
+    o.place = (int*)(base + b_rec + b_list + b_sorted);
+    o.cell = list;
+    o.buckets = buckets;
+    o.jumps = (unsigned*)(zero + sizeof(RunState));
+    if (ptype == HD_F64)
+      launch_chained(k_points_cell<double>, blocks_for(n, 256), 256, 0, s, bvh_dev(B), (const double*)Pts, n, o);
+    else
+      launch_chained(k_points_cell<float>, blocks_for(n, 256), 256, 0, s, bvh_dev(B), (const float*)Pts, n, o);
+    launch_chained(k_points_scan, 1, 1024, 0, s, o, n);
+    launch_chained(k_points_place, blocks_for(n, 256), 256, 0, s, o, n);
+  }
   if (ptype == HD_F64)
-    launch_chained(k_points_in<P, double>, blocks_for(n, 256), 256, 0, s, (const double*)Pts, n, tmp);
+    launch_chained(k_points_in<P, double>, blocks_for(n, 256), 256, 0, s, (const double*)Pts, n, tmp, o);
   else
-    launch_chained(k_points_in<P, float>, blocks_for(n, 256), 256, 0, s, (const float*)Pts, n, tmp);
+    launch_chained(k_points_in<P, float>, blocks_for(n, 256), 256, 0, s, (const float*)Pts, n, tmp, o);
   {
     TraceScope tr(HD_K_QUERY, s);
     query_points<P>(bvh_dev(B), tmp, n, st, list, s, sorted, buckets);
   }
-  launch_chained(k_points_out<P>, blocks_for(n, 256), 256, 0, s, tmp, n, B->tri_vid, dist, idx, foot, dlo);
-  HD_TRY_LAUNCH();
-  HD_TRY(cudaFreeAsync(tmp, s));
-  HD_TRY(cudaFreeAsync(st, s));
-  if (list) HD_TRY(cudaFreeAsync(list, s));
-  if (sorted) HD_TRY(cudaFreeAsync(sorted, s));
-  if (buckets) HD_TRY(cudaFreeAsync(buckets, s));
+  launch_chained(k_points_out<P>, blocks_for(n, 256), 256, 0, s, (const typename P::Vtx*)tmp, n, (const int4*)B->tri_vid,
+                 dist, idx, foot, dlo, o);
+  e = cudaGetLastError();
+  const cudaError_t f = cudaFreeAsync(base, s);
+  HD_TRY(e);
+  HD_TRY(f);
   return HD_OK;
 }
 

@@ -43,16 +43,23 @@ constexpr int kCoopWarps = 4;              // warps per block of k_query_long
 #ifndef HD_COOP_MIN_BLOCKS
 #define HD_COOP_MIN_BLOCKS 12
 #endif
-// resident blocks per SM asked of the compiler: 12 blocks of 4 warps (<= 40 registers, a few
-// values spilled to L1; 10 KB of stacks each).  The traversal waits on dependent node fetches,
-// so warps in flight pay: on the large soup's long queries, blocks x stack entries of 6 x 768,
-// 8 x 512, 10 x 384, 12 x 320 and 16 x 256 took 2.03, 1.86, 1.70, 1.67 and 1.80 ms per call.
+// resident blocks per SM asked of the compiler, for a kernel that never cuts: 12 blocks of 4
+// warps (<= 40 registers, a few values spilled to L1; 10 KB of stacks each).  The traversal
+// waits on dependent node fetches, so warps in flight pay: on the batch of 128 pairs 7, 8, 9,
+// 10, 12 blocks took 7.53, 6.80, 6.48, 6.29, 6.19 ms.  With cuts (HD_COOP_MIN_BLOCKS_CUT) the
+// kernel holds a second traversal and most queries end after a few nodes, so spills cost more
+// than the warps bring: 8, 9, 10, 12 blocks took 0.385, 0.391, 0.403, 0.422 ms on the large
+// soup and 3.49, 3.56, 3.62, 3.73 ms on the slivers.
 constexpr int kCoopMinBlocks = HD_COOP_MIN_BLOCKS;
+#ifndef HD_COOP_MIN_BLOCKS_CUT
+#define HD_COOP_MIN_BLOCKS_CUT 8
+#endif
+constexpr int kCoopMinBlocksCut = HD_COOP_MIN_BLOCKS_CUT;
 // The FP64 policy's cooperative traversal keeps doubles in flight (its query point, the best
 // squared distance and closest point, the triangle being tested): at 40 registers it spills
 // heavily, so it asks for fewer blocks per SM, and its lanes keep their queries longer.
 #ifndef HD_COOP_MIN_BLOCKS_D
-#define HD_COOP_MIN_BLOCKS_D 6
+#define HD_COOP_MIN_BLOCKS_D 4
 #endif
 #ifndef HD_LONG_BUDGET_D
 #define HD_LONG_BUDGET_D 10

@@ -535,6 +535,12 @@ __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const dou
 
 // ----------------------------------------------------------------------------- the policy
 
+#ifndef HD_FP64_SPREAD
+#define HD_FP64_SPREAD 8
+#endif
+#ifndef HD_FP64_SPREAD_BOUNDS
+#define HD_FP64_SPREAD_BOUNDS 3
+#endif
 #ifndef HD_FP64_BOUND_REGS
 #define HD_FP64_BOUND_REGS 128
 #endif
@@ -547,8 +553,11 @@ struct PolicyD {
   using Item = ItemD;
   using UT = double;
   static constexpr bool kFp64 = true;
-  static constexpr int kCoopBlocks = HD_COOP_MIN_BLOCKS_D;  // resident blocks per SM of the cooperative traversal
+  // resident blocks per SM of the cooperative traversal, with cuts / without
+  static constexpr int kCoopBlocksCut = HD_COOP_MIN_BLOCKS_D, kCoopBlocks = HD_COOP_MIN_BLOCKS_D;
   static constexpr int kLongBudget = HD_LONG_BUDGET_D;      // triangle tests of a lane before the hand-off
+  // warps per SM that a short list of queries / of bounds is spread over (spread_lanes)
+  static constexpr int kSpread = HD_FP64_SPREAD, kSpreadBounds = HD_FP64_SPREAD_BOUNDS;
   static constexpr int kBoundRegs = HD_FP64_BOUND_REGS;  // register cap of the UpperBound kernels
   static constexpr int kPaperRegs = HD_FP64_PAPER_REGS;  // ... of their paper-order instantiation
 

@@ -489,6 +489,9 @@ __device__ inline float upper_bound_m_paper(const BvhDev& B, const VM t[3], floa
 
 // ----------------------------------------------------------------------------- the policy
 
+#ifndef HD_MIXED_SPREAD
+#define HD_MIXED_SPREAD 8
+#endif
 #ifndef HD_MIXED_BOUND_REGS
 #define HD_MIXED_BOUND_REGS 96
 #endif
@@ -501,8 +504,11 @@ struct PolicyM {
   using Item = ItemM;
   using UT = float;
   static constexpr bool kFp64 = false;
-  static constexpr int kCoopBlocks = kCoopMinBlocks;  // resident blocks per SM of the cooperative traversal
+  // resident blocks per SM of the cooperative traversal, with cuts / without
+  static constexpr int kCoopBlocksCut = kCoopMinBlocksCut, kCoopBlocks = kCoopMinBlocks;
   static constexpr int kLongBudget = ::hd::kLongBudget;  // triangle tests of a lane before the hand-off
+  // warps per SM that a short list of queries / of bounds is spread over (spread_lanes)
+  static constexpr int kSpread = HD_MIXED_SPREAD, kSpreadBounds = HD_MIXED_SPREAD;
   static constexpr int kBoundRegs = HD_MIXED_BOUND_REGS;  // register cap of the UpperBound kernels
   static constexpr int kPaperRegs = HD_MIXED_PAPER_REGS;  // ... of their paper-order instantiation
 

@@ -65,11 +65,12 @@ int run(const hd_bvh* B, const void* Pts, int ptype, int64_t n, cudaStream_t s, 
   int* list = (int*)((unsigned char*)base + kNoAllocMaxPoints * 64 + kNoAllocTail);
   HD_TRY(cudaMemsetAsync(st, 0, sizeof(RunState), s));  // counters start at zero every call
   if (ptype == HD_F64)
-    k_points_in<P, double><<<blocks_for(n, 256), 256, 0, s>>>((const double*)Pts, n, rec);
+    launch_chained(k_points_in<P, double>, blocks_for(n, 256), 256, 0, s, (const double*)Pts, n, rec, PointOrder{});
   else
-    k_points_in<P, float><<<blocks_for(n, 256), 256, 0, s>>>((const float*)Pts, n, rec);
+    launch_chained(k_points_in<P, float>, blocks_for(n, 256), 256, 0, s, (const float*)Pts, n, rec, PointOrder{});
   query_points<P>(bvh_dev(B), rec, n, st, list, s);
-  k_points_out<P><<<blocks_for(n, 256), 256, 0, s>>>(rec, n, B->tri_vid, dist, idx, foot, dlo);
+  launch_chained(k_points_out<P>, blocks_for(n, 256), 256, 0, s, (const typename P::Vtx*)rec, n,
+                 (const int4*)B->tri_vid, dist, idx, foot, dlo, PointOrder{});
   HD_TRY_LAUNCH();
   return HD_OK;
 }
