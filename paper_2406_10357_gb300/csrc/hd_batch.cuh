@@ -551,7 +551,8 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
         const PairLevel<P> pl = pair_level<P>(x, p);
         int code;
         const typename P::UT U =
-            P::paper_u3(x.pd[p].B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], pl.lv.lf, pl.rp, e.u12, code, ty.c);
+            P::paper_u3(x.pd[p].B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], pl.lv.lf, pl.rp, e.u12, e.up,
+                        code, ty.c);
         it.U = e.up < U ? e.up : U;
         classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
       }

@@ -799,7 +799,7 @@ __device__ inline void bound_rebin(const BvhDev& B, const typename P::Vtx* pool,
         it.v[1] = e.v[1];
         it.v[2] = e.v[2];
         int code;
-        const typename P::UT U = P::paper_u3(B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], lv.lf, rp, e.u12, code, c);
+        const typename P::UT U = P::paper_u3(B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], lv.lf, rp, e.u12, e.up, code, c);
         it.U = e.up < U ? e.up : U;
         classify<P>(st, it, lv.th, code, next, next_cap, u4list, ty);
       }

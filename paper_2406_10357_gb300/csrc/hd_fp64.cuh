@@ -714,7 +714,7 @@ struct PolicyD {
     UT U;
     float u12;
     if (!paper_cheap(B, a, b, c, lf, rp, &U, &code, &u12)) return U;
-    return paper_u3(B, a, b, c, lf, rp, u12, code, cnt);
+    return paper_u3(B, a, b, c, lf, rp, u12, INFINITY, code, cnt);
   }
   __device__ static bool paper_cheap(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf,
                                      const RunParams& rp, UT* U, int* code, float* u12) {
@@ -743,7 +743,7 @@ struct PolicyD {
     return true;
   }
   __device__ static UT paper_u3(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf, const RunParams& rp,
-                                float, int& code, Counters& cnt) {
+                                float, float, int& code, Counters& cnt) {
     VM t[3];
     vertices_m(a, b, c, t);
     const float lim = filter_limit(B, t, lf, rp);
