@@ -104,9 +104,9 @@ enum {
  * runs on host threads with one stream each, instead of the default batched run in which every
  * kernel launch works on the items of all pairs. */
 /* HD_FLAG_NO_SMALL_ROUNDS: every frontier round runs as a sequence of grid-wide kernels.  By
- * default, rounds over a frontier of at most 64 items (the last rounds of most runs) run
- * inside one single-block kernel that loops over them without the host; the results are the
- * same either way. */
+ * default, rounds over a small frontier (at most a few hundred items: the last rounds of most
+ * runs) run inside one kernel, a single thread-block cluster, that loops over them without
+ * the host; the results are the same either way. */
 /* HD_FLAG_WELD_B (read by hd_build_B, for the mesh it builds a BVH of; for
  * hd_hausdorff_sym give it when building A's BVH too): vertices at exactly the same
  * position get one id before the adjacency
@@ -291,7 +291,7 @@ int hd_upper_bounds(const hd_bvh* B, const double* T, const double* Td, const in
  * the number of launches and their total device time in milliseconds.  Each pair costs a
  * few microseconds of host time.  Kinds: the whole BVH build of one hd_build_B call
  * (counted as one launch), the nearest-triangle lane traversal (k_query), UpperBound of
- * faces and children, select/split/compaction, validation/pool set-up, the single-block
+ * faces and children, select/split/compaction, validation/pool set-up, the single-cluster
  * kernel that runs whole rounds over small frontiers, and the warp-cooperative traversal of
  * long queries (k_query_long). */
 enum { HD_K_BUILD = 0, HD_K_QUERY = 1, HD_K_BOUND = 2, HD_K_SELECT = 3, HD_K_PREP = 4, HD_K_SMALL = 5, HD_K_LONG = 6,

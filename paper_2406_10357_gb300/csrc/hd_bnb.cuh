@@ -1239,22 +1239,37 @@ static __global__ void k_round_ctl(RunState* st, RoundCtl c, int init, int n_poo
 
 // ----------------------------------------------------------------------------- small rounds
 
-// Rounds over a small frontier (the last rounds of most runs) in one block: each phase of a
-// round is a kernel of the normal path, and for a frontier of a few dozen items each is one
-// pass of a few warps, so the launches and the host's reading of the round dominate.  Here
-// one block runs the same steps (control, select, query, cooperative query, bound, u4) with
-// block barriers between them, round after round, until the loop stops, the frontier grows
-// past kTailFront, or a round hands more than kTailWarps queries to the cooperative pass (a
-// round with many long traversals needs the whole GPU); the normal path then takes over, so
-// any frontier is correct.
+// Rounds over a small frontier (the last rounds of most runs) in one cluster of blocks: each
+// phase of a round is a kernel of the normal path, and for a frontier of a few hundred items
+// each is one pass of a few warps, so the launches and the host's reading of the round
+// dominate.  Here one cluster runs the same steps (control, select, query, cooperative query,
+// bound, second pass) with cluster barriers between them, round after round, until the loop
+// stops, the frontier grows past P::kTailFront, or a round hands more than kTailLong queries to
+// the cooperative pass (a round with many long traversals needs the whole GPU); the normal
+// path then takes over, so any frontier is correct.  The phases take their work from the same
+// counters whatever the number of blocks; one block of 256 threads ran these rounds before
+// (last rounds of the 320-triangle spheres in FP64 0.108 -> 0.093 ms, of the two-sided scan
+// 0.175 -> 0.146 ms).  A MIXED pair of 320 triangles took 421, 426, 377, 383 us with a
+// frontier of at most 64, 256, 512, 1024 items, larger pairs the same with any; an FP64 one
+// 691, 707, 901, 905 us: eight SMs' FP64 pipes are too few for more than the smallest rounds.
 constexpr int kTailThreads = 256;
 constexpr int kTailWarps = kTailThreads / 32;
+#ifndef HD_TAIL_CLUSTER
+#define HD_TAIL_CLUSTER 8
+#endif
+constexpr int kTailCluster = HD_TAIL_CLUSTER;  // blocks (8: the largest portable cluster)
 #ifndef HD_TAIL_LONG
-#define HD_TAIL_LONG kTailWarps
+#define HD_TAIL_LONG (kTailCluster * kTailWarps)
 #endif
 constexpr int kTailLong = HD_TAIL_LONG;  // most long queries a round may hand off and stay in the small-round kernel
-constexpr int kTailFront = 64;
 constexpr size_t kTailSmem = (sizeof(unsigned) + sizeof(float)) * kTailWarps * kCoopStack;
+
+// Every thread of the cluster; global writes before it are seen by every block after it.
+__device__ inline void tail_sync() {
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  __threadfence();
+}
 
 template <class P>
 struct TailBufs {
@@ -1271,42 +1286,40 @@ struct TailBufs {
 };
 
 template <class P>
-__global__ void __launch_bounds__(kTailThreads) k_tail_rounds(BvhDev B, TailBufs<P> a, RunState* st, RunParams rp,
-                                                              RoundCtl c, int init, int n_pool0, int cur) {
+__global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThreads)
+    k_tail_rounds(BvhDev B, TailBufs<P> a, RunState* st, RunParams rp, RoundCtl c, int init, int n_pool0, int cur) {
   extern __shared__ __align__(16) unsigned char tail_smem[];  // kTailSmem bytes: the warps' cooperative stacks
   unsigned* s_code = reinterpret_cast<unsigned*>(tail_smem);
   float* s_e = reinterpret_cast<float*>(tail_smem + sizeof(unsigned) * kTailWarps * kCoopStack);
-  __shared__ int s_go;
   grid_dep_wait();
   grid_dep_launch();
+  const bool first = blockIdx.x == 0 && threadIdx.x == 0;
   // a round here hands off at most a few queries: the list keeps its order
   const LongList lq = {a.longq.idx, a.longq.cap, nullptr, nullptr};
   int rounds = 0;
   for (;;) {
-    if (threadIdx.x == 0) {
-      // the control step of k_round_ctl, refusing to open a round over kTailFront items
-      round_ctl_body(st, c, init, n_pool0, kTailFront, kTailLong);
-      s_go = !st->stop && st->in_round;
-    }
+    // the control step of k_round_ctl, refusing to open a round over P::kTailFront items
+    if (first) round_ctl_body(st, c, init, n_pool0, P::kTailFront, kTailLong);
     init = 0;
-    __syncthreads();
-    if (!s_go) break;
+    tail_sync();
+    // the same for every thread of the cluster: only the control step writes these
+    if (*(volatile int*)&st->stop || !*(volatile int*)&st->in_round) break;
     select_body<P>(a.front[cur], st, rp, a.split_par, a.split_mid, a.tab, a.pool, a.front[cur ^ 1], a.front_cap,
                    a.promo, a.promo_cap);
-    __syncthreads();
+    tail_sync();
     query_body<P>(B, a.pool, 0, nullptr, 3, 0, st, rp.slack, rp.dyn, true, a.tab, lq);
-    __syncthreads();
+    tail_sync();
     query_long_body<P, true>(B, a.pool, lq, st, rp.slack, rp.dyn, true, s_code, s_e);
-    __syncthreads();
+    tail_sync();
     typename P::Item* left = a.u4list ? a.u4list : a.front[cur];
     bound_children_body<P>(B, a.pool, a.split_par, a.split_mid, st, rp, a.front[cur ^ 1], a.front_cap, left);
-    __syncthreads();
+    tail_sync();
     bound_u4_body<P>(B, a.pool, left, a.front_cap, st, rp, a.front[cur ^ 1], a.front_cap);
-    __syncthreads();
+    tail_sync();
     cur ^= 1;
     ++rounds;
   }
-  if (threadIdx.x == 0) st->tail_rounds = rounds;
+  if (first) st->tail_rounds = rounds;
 }
 
 // Nearest queries for external points (hd_nearest): P as double rows.
@@ -1648,6 +1661,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
                  grid_b = persistent_grid_bs(k_children, bs, grid_b_cache[paper ? 1 : 0], smem_b);
   const bool cuts = cut_enabled(o);
   int64_t front_bound = first_front_bound;  // the first round is queued without a wait
+  int last_long = -1;  // long queries of the last round read (-1: none read yet)
   int cur = R.cur;
   bool init = true;
   // the run state and parameters after the work queued so far, into ring slot `slot`
@@ -1678,7 +1692,9 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     }
     {
       TraceScope tr(HD_K_LONG, s);
-      sort_long<P>(B, R.pool, R.longq, st, true, sms, s, rp.dyn);
+      // The reordering where this round may hand off a list worth it: not where the last round
+      // read handed off few, of a frontier at least a quarter of this one's bound.
+      if (last_long < 0 || 8 * (int64_t)last_long >= kSortMin) sort_long<P>(B, R.pool, R.longq, st, true, sms, s, rp.dyn);
       launch_query_long<P>(cuts, B, R.pool, R.longq, st, rp.slack, rp.dyn, true, s);
     }
     {
@@ -1692,7 +1708,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     cur ^= 1;
     return snapshot(slot);
   };
-  // the small-round kernel, for a frontier of at most kTailFront items; it may run any number
+  // the small-round kernel, for a frontier of at most P::kTailFront items; it may run any number
   // of rounds, so nothing is queued after it until its snapshot has been read
   const TailBufs<P> tb = {{R.front[0], R.front[1]}, R.split_par, R.split_mid, R.tab, R.pool, R.promo, (int)R.promo_cap,
                           (int)R.front_cap, R.u4list, R.longq};
@@ -1700,19 +1716,18 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     HD_TRY(tail_smem_attr<P>());
     {
       TraceScope tr(HD_K_SMALL, s);
-      launch_chained(k_tail_rounds<P>, 1, kTailThreads, kTailSmem, s, B, tb, st, rp, c, init ? 1 : 0, n_pool0, cur);
+      launch_chained(k_tail_rounds<P>, kTailCluster, kTailThreads, kTailSmem, s, B, tb, st, rp, c, init ? 1 : 0, n_pool0, cur);
       init = false;
     }
     HD_TRY_LAUNCH();
     return snapshot(slot);
   };
   long long issued = 0, seen = 0, tail_at = -1;  // tail_at: the snapshot of the small-round kernel in flight
-  int last_long = 0;  // long queries of the last round read
   for (;;) {
     const long long ahead = seen >= HD_AHEAD_FROM ? 2 : 1;  // rounds in flight, the one being read included
     while (issued < seen + ahead && tail_at < 0) {
       int rc;
-      if (front_bound <= kTailFront && last_long <= kTailLong && !(o.flags & HD_FLAG_NO_SMALL_ROUNDS)) {
+      if (front_bound <= P::kTailFront && last_long <= kTailLong && !(o.flags & HD_FLAG_NO_SMALL_ROUNDS)) {
         rc = issue_tail((int)(issued & 1));
         tail_at = issued;
       } else {

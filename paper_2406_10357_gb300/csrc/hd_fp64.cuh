@@ -556,6 +556,7 @@ struct PolicyD {
   // resident blocks per SM of the cooperative traversal, with cuts / without
   static constexpr int kCoopBlocksCut = HD_COOP_MIN_BLOCKS_D, kCoopBlocks = HD_COOP_MIN_BLOCKS_D;
   static constexpr int kLongBudget = HD_LONG_BUDGET_D;      // triangle tests of a lane before the hand-off
+  static constexpr int kTailFront = 64;  // largest frontier of the small-round kernel
   // warps per SM that a short list of queries / of bounds is spread over (spread_lanes)
   static constexpr int kSpread = HD_FP64_SPREAD, kSpreadBounds = HD_FP64_SPREAD_BOUNDS;
   static constexpr int kBoundRegs = HD_FP64_BOUND_REGS;  // register cap of the UpperBound kernels

@@ -539,6 +539,7 @@ struct PolicyM {
   // resident blocks per SM of the cooperative traversal, with cuts / without
   static constexpr int kCoopBlocksCut = kCoopMinBlocksCut, kCoopBlocks = kCoopMinBlocks;
   static constexpr int kLongBudget = ::hd::kLongBudget;  // triangle tests of a lane before the hand-off
+  static constexpr int kTailFront = 512;  // largest frontier of the small-round kernel
   // warps per SM that a short list of queries / of bounds is spread over (spread_lanes)
   static constexpr int kSpread = HD_MIXED_SPREAD, kSpreadBounds = HD_MIXED_SPREAD;
   static constexpr int kBoundRegs = HD_MIXED_BOUND_REGS;  // register cap of the UpperBound kernels
