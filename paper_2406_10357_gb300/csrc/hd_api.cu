@@ -148,31 +148,33 @@ int nearest_points_mixed(const hd_bvh* B, const void* Pts, int ptype, int64_t n,
 int upper_bounds_mixed(const hd_bvh* B, const double* T, const double* Td, const int32_t* TI, const double* Tq,
                        int64_t n, double l, const RunParams& rp, cudaStream_t s, double* U, int32_t* code);
 
+// Launched with whole warps: lanes past the last triangle take part in the votes of ub_u3.
 __global__ void k_upper_bounds(BvhDev B, const int* inv, const double* T, const double* Td, const int32_t* TI,
                                const double* Tq, int64_t n, double l, RunParams rp, double* U, int32_t* code) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool on = i < n;
   VI t[3];
+  double own[3] = {0.0, 0.0, 0.0};
   for (int k = 0; k < 3; ++k) {
+    t[k] = {{0.0, 0.0, 0.0}, 0.0, 0, {0.0, 0.0, 0.0}};
+    if (i >= n) continue;
     const double* v = T + 9 * i + 3 * k;
     const double* q = Tq + 9 * i + 3 * k;
-    int I = TI[3 * i + k];
+    const int I = TI[3 * i + k];
     if (I < 0 || I >= B.nF) {  // not a triangle of B: no bound
-      U[i] = NAN;
-      code[i] = -1;
-      return;
+      on = false;
+      continue;
     }
     t[k] = {{v[0], v[1], v[2]}, Td[3 * i + k], inv[I], {q[0], q[1], q[2]}};
+    D3 x;  // the distances given need not be those to the triangles given
+    own[k] = sqrt(tri_dist2(B.tri64, B.tri32, t[k].I, t[k].v, x));
   }
   unsigned ev = 0;
   int c;
-  double own[3];  // the distances given need not be those to the triangles given
-  for (int k = 0; k < 3; ++k) {
-    D3 x;
-    own[k] = sqrt(tri_dist2(B.tri64, B.tri32, t[k].I, t[k].v, x));
-  }
-  U[i] = upper_bound_d(B, t, own, l, rp.order, rp.n_bounds, true, c, ev);
-  code[i] = c;
+  const double u = upper_bound_d(B, t, own, l, rp.order, rp.n_bounds, true, on, c, ev);
+  if (i >= n) return;
+  U[i] = on ? u : NAN;
+  code[i] = on ? c : -1;
 }
 
 }  // namespace hd

@@ -657,14 +657,17 @@ __global__ void k_batch_bound_u4(BatchCtx x, const typename P::Vtx* pool, const 
     const int64_t t = base + (threadIdx.x & 31);
     int p = -1;
     PairDelta<P> ty;
-    if (t < n) {
-      p = u4_pair[t];
-      typename P::Item it = u4list[t];
+    const bool on = t < n;
+    if (P::kPassVotes || on) {
+      // (lanes without an item take part in the votes, with the warp's first item)
+      p = u4_pair[on ? t : base];
+      typename P::Item it = u4list[on ? t : base];
       const PairLevel<P> pl = pair_level<P>(x, p);
       int code;
-      P::bound_deferred(x.pd[p].B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], pl.lv.l, pl.lv.th.lo, pl.rp, it.U, code,
-                        ty.c);
-      classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, nullptr, nullptr, ty);
+      P::bound_deferred(x.pd[p].B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], on, pl.lv.l, pl.lv.th.lo, pl.rp, it.U,
+                        code, ty.c);
+      if (on) classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, nullptr, nullptr, ty);
+      else p = -1;
     }
     acc_batch(acc, x.sts, p, ty);
   }

@@ -875,11 +875,13 @@ __device__ inline void bound_u4_body(BvhDev B, const typename P::Vtx* pool, cons
   for (int64_t base = (blockIdx.x * (int64_t)wpb + (threadIdx.x >> 5)) * lanes; base < n;
        base += (int64_t)gridDim.x * wpb * lanes) {
     const int64_t t = base + lane;
-    if (lane >= lanes || t >= n) continue;
-    typename P::Item it = u4list[t];
+    const bool on = lane < lanes && t < n;
+    if (!P::kPassVotes && !on) continue;
+    // (lanes without an item take part in the votes, with the warp's first item)
+    typename P::Item it = u4list[on ? t : base];
     int code;
-    P::bound_deferred(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.l, th.lo, rp, it.U, code, c);
-    classify<P>(st, it, th, code, next, next_cap, nullptr, ty);
+    P::bound_deferred(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], on, lv.l, th.lo, rp, it.U, code, c);
+    if (on) classify<P>(st, it, th, code, next, next_cap, nullptr, ty);
   }
   if constexpr (P::kFp64) flush_counters(st, c);
   flush_tally(st, ty);

@@ -337,20 +337,18 @@ __device__ inline D3 tri_vertex(const BvhDev& B, int j, int slot) {
   return {v.x, v.y, v.z};
 }
 
-// Distance from x to triangle j of B, where it may exceed h: an FP32 upper bound of it (pt_hi)
-// first, and the FP64 distance only if that does not settle the comparison.
-__device__ inline void raise_dist(const BvhDev& B, int j, D3 x, double& h, unsigned& evals) {
-  FFP P;
-  P.h = {__double2float_rn(x.x), __double2float_rn(x.y), __double2float_rn(x.z)};
-  P.l = {__double2float_rn(x.x - (double)P.h.x), __double2float_rn(x.y - (double)P.h.y),
-         __double2float_rn(x.z - (double)P.h.z)};
-  const float4* t = B.tri32 + 3 * (size_t)j;
-  // the float forms of B and x, and the FP64 rounding (NearestD::guard)
-  const float guard = __fmaf_ru(0x1p-39f, amax3(P.h), __fadd_ru(__ldg(B.meta), 1e-37f));
-  ++evals;
-  if (__fadd_ru(pt_hi(P, __ldg(t), __ldg(t + 1), __ldg(t + 2)), guard) <= __double2float_rd(h)) return;
-  D3 q;
-  h = fmax(h, sqrt(tri_dist2(B.tri64, B.tri32, j, x, q)));
+// v as a vertex of the certified FP32 bounds: its position as a float pair, its distance
+// rounded up.
+__device__ inline VM vertex_m(D3 v, double d, int I) {
+  VM m;
+  m.p.h = {__double2float_rn(v.x), __double2float_rn(v.y), __double2float_rn(v.z)};
+  m.p.l = {__double2float_rn(v.x - (double)m.p.h.x), __double2float_rn(v.y - (double)m.p.h.y),
+           __double2float_rn(v.z - (double)m.p.h.z)};
+  m.dhi = __double2float_ru(d);
+  m.I = I;
+  m.q = {0.f, 0.f, 0.f};
+  m.qerr = 0.f;
+  return m;
 }
 
 // Eq. (uexact): the three vertices are nearest to one triangle S; h(T,S) = max_i |v_i - q_i|.
@@ -389,73 +387,153 @@ __device__ inline double ub_u2(const VI t[3], const EdgesD& E, double cap) {
 }
 
 // Kang et al. 2018 bound, Eqs. (Kang2018_case1) and (Kang2018_case2).  own[i] = d(v_i, S_i).
+// Must be called by all 32 lanes of the warp; lanes with on == false only vote.
+//
 // Every term is a maximum of point-triangle distances, so a distance is computed in FP64 only
-// where its FP32 upper bound exceeds the maximum so far (raise_dist); a maximum that
-// can no longer lower the minimum it enters is abandoned.  The loops are not unrolled: one
-// copy of the FP64 test per loop keeps the kernel within the instruction cache.
-__device__ inline double ub_u3(const BvhDev& B, const VI t[3], const double own[3], double cap, unsigned& evals) {
-  int lone = -1;
-  if (!(t[0].I == t[1].I && t[1].I == t[2].I)) {
-    if (t[1].I == t[2].I) lone = 0;
-    else if (t[0].I == t[2].I) lone = 1;
-    else if (t[0].I == t[1].I) lone = 2;
-  }
-  int fs0, fs1, fo, go;
-  // v1 is the vertex alone on its triangle (selected by branches: no runtime array index)
-  VI v1 = t[0], v2 = t[1], v3 = t[2];
-  if (lone == 1) { v1 = t[1]; v2 = t[2]; v3 = t[0]; }
-  else if (lone == 2) { v1 = t[2]; v2 = t[0]; v3 = t[1]; }
+// where its FP32 upper bound exceeds the maximum so far, and a maximum that can no longer
+// lower the minimum it enters is abandoned.  Few of the 4 (case 1) or 15 (case 2) distances
+// are left then, at different places for each lane; so a lane goes through them until one
+// needs FP64, waits, and the waiting lanes run the FP64 test together.  (Tested where they
+// occur, some lane needs FP64 at almost every place, and the warp pays for each: the pass had
+// 9 to 15 lanes active.  Bounds of the batch of 32 small pairs in FP64 4.34 -> 3.55 ms, of the
+// torus pair 0.418 -> 0.376 ms.)
+__device__ inline double ub_u3(const BvhDev& B, const VI t[3], const double own[3], double cap, bool on, unsigned& evals) {
   const double dmax = fmax(own[0], fmax(own[1], own[2]));
-  if (lone >= 0 && shared_edge(B, v1.I, v2.I, fs0, fs1, fo, go)) {
-    int S1 = v1.I, S2 = v2.I;
-    D3 p0 = tri_vertex(B, S1, fs0), e = tri_vertex(B, S1, fs1) - p0;
-    D3 b1 = 0.5 * (v1.v + v2.v), b2 = 0.5 * (v1.v + v3.v);
-    double el = len(e);
-    if (el > 0.0) {
-      D3 eh = (1.0 / el) * e;
-      D3 a1 = tri_vertex(B, S1, fo) - p0, a2 = tri_vertex(B, S2, go) - p0;
-      D3 w1 = a1 - dot(a1, eh) * eh, w2 = a2 - dot(a2, eh) * eh;
-      double n1 = len(w1), n2 = len(w2);
-      if (n1 > 0.0 && n2 > 0.0) {
-        D3 nb = (1.0 / n1) * w1 - (1.0 / n2) * w2;
-        double s1 = dot(nb, v1.v - p0), s2 = dot(nb, v2.v - p0), s3 = dot(nb, v3.v - p0);
-        if (s1 >= 0.0 && s2 <= 0.0 && s3 <= 0.0 && s1 - s2 > 0.0 && s1 - s3 > 0.0) {
-          b1 = v1.v + (s1 / (s1 - s2)) * (v2.v - v1.v);
-          b2 = v1.v + (s1 / (s1 - s3)) * (v3.v - v1.v);
+  // the distances to take, in order: case 1 (c1): the split points b1, b2 against S1, then S2
+  // (v1 against S1 and v2, v3 against S2 are the vertices' own); case 2: steps 0..5 the two
+  // other vertices against S_i, then 6..14 the quadrilaterals (v_i, m_i, b, m_{i-1}) against S_i
+  int k = 0, kend = 0, S1 = 0, S2 = 0;
+  bool c1 = false;
+  D3 b1 = t[0].v, b2 = t[0].v;
+  double h = own[0], best = cap;
+  VM f[3];
+  FFP fb1, fb2, fm[3], fbc;
+  float bm[3] = {0.f, 0.f, 0.f}, bb = 0.f, guard = 0.f;
+  if (on) {
+    int lone = -1;
+    if (!(t[0].I == t[1].I && t[1].I == t[2].I)) {
+      if (t[1].I == t[2].I) lone = 0;
+      else if (t[0].I == t[2].I) lone = 1;
+      else if (t[0].I == t[1].I) lone = 2;
+    }
+    int fs0, fs1, fo, go;
+    // v1 is the vertex alone on its triangle (selected by branches: no runtime array index)
+    VI v1 = t[0], v2 = t[1], v3 = t[2];
+    if (lone == 1) { v1 = t[1]; v2 = t[2]; v3 = t[0]; }
+    else if (lone == 2) { v1 = t[2]; v2 = t[0]; v3 = t[1]; }
+    c1 = lone >= 0 && shared_edge(B, v1.I, v2.I, fs0, fs1, fo, go);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[i] = vertex_m(t[i].v, 0.0, t[i].I);
+    // the float forms of B and the points, and the FP64 rounding (NearestD::guard)
+    const float pmax = fmaxf(amax3(f[0].p.h), fmaxf(amax3(f[1].p.h), amax3(f[2].p.h)));
+    guard = __fmaf_ru(0x1p-38f, pmax, __fadd_ru(__ldg(B.meta), 1e-37f));
+    if (c1) {
+      S1 = v1.I;
+      S2 = v2.I;
+      D3 p0 = tri_vertex(B, S1, fs0), e = tri_vertex(B, S1, fs1) - p0;
+      b1 = 0.5 * (v1.v + v2.v);
+      b2 = 0.5 * (v1.v + v3.v);
+      double el = len(e);
+      if (el > 0.0) {
+        D3 eh = (1.0 / el) * e;
+        D3 a1 = tri_vertex(B, S1, fo) - p0, a2 = tri_vertex(B, S2, go) - p0;
+        D3 w1 = a1 - dot(a1, eh) * eh, w2 = a2 - dot(a2, eh) * eh;
+        double n1 = len(w1), n2 = len(w2);
+        if (n1 > 0.0 && n2 > 0.0) {
+          D3 nb = (1.0 / n1) * w1 - (1.0 / n2) * w2;
+          double s1 = dot(nb, v1.v - p0), s2 = dot(nb, v2.v - p0), s3 = dot(nb, v3.v - p0);
+          if (s1 >= 0.0 && s2 <= 0.0 && s3 <= 0.0 && s1 - s2 > 0.0 && s1 - s3 > 0.0) {
+            b1 = v1.v + (s1 / (s1 - s2)) * (v2.v - v1.v);
+            b2 = v1.v + (s1 / (s1 - s3)) * (v3.v - v1.v);
+          }
         }
       }
+      fb1 = vertex_m(b1, 0.0, 0).p;
+      fb2 = vertex_m(b2, 0.0, 0).p;
+      h = dmax;
+      kend = 4;
+    } else {
+      const F3 e01 = edge(f[0], f[1]), e02 = edge(f[0], f[2]), e12 = edge(f[1], f[2]);
+      fm[0] = along(f[0], e01, 0.5f, bm[0]);
+      fm[1] = along(f[1], e12, 0.5f, bm[1]);
+      fm[2] = along(f[0], e02, 0.5f, bm[2]);
+      fbc = along(f[0], e01 + e02, 1.f / 3.f, bb);
+      bb = __fmul_ru(16.f * kU, fmaxf(amax3(e01), fmaxf(amax3(e02), amax3(f[0].p.l))));
+      kend = 15;
     }
-    // v1 against S1, v2 and v3 against S2 are the vertices' own; the split points against both
-    double h = dmax;
-#pragma unroll 1
-    for (int k = 0; k < 4 && h < cap; ++k) raise_dist(B, k < 2 ? S1 : S2, (k & 1) ? b2 : b1, h, evals);
-    return h;
   }
-  // min over the triangles of the largest vertex distance to each
-  double best = cap;
-#pragma unroll 1
-  for (int k = 0; k < 3; ++k) {
-    const int S = k == 0 ? t[0].I : k == 1 ? t[1].I : t[2].I;
-    const D3 x = k == 0 ? t[1].v : k == 1 ? t[2].v : t[0].v, y = k == 0 ? t[2].v : k == 1 ? t[0].v : t[1].v;
-    double h = k == 0 ? own[0] : k == 1 ? own[1] : own[2];
-#pragma unroll 1
-    for (int j = 0; j < 2 && h < best; ++j) raise_dist(B, S, j ? y : x, h, evals);
-    best = fmin(best, h);
+  // step k is settled: on to the next one (and the next maximum of case 2)
+  auto next = [&]() {
+    ++k;
+    if (!c1 && k <= 6 && (k & 1) == 0) {
+      best = fmin(best, h);
+      h = k == 2 ? own[1] : k == 4 ? own[2] : dmax;
+    }
+  };
+  bool pend = false;
+  int S = 0, i = 0, j = 0;
+  for (;;) {
+    while (k < kend && !pend) {
+      if (c1) {
+        if (!(h < cap)) {
+          k = kend;
+          break;
+        }
+        S = k < 2 ? S1 : S2;
+      } else {
+        if (!(h < best)) {  // this maximum cannot lower the minimum
+          if (k < 6) {
+            k |= 1;
+            next();
+            continue;
+          }
+          k = kend;
+          break;
+        }
+        const int r = k < 6 ? k : k - 6;
+        i = k < 6 ? r >> 1 : r / 3;
+        j = k < 6 ? r & 1 : r - 3 * i;
+        S = i == 0 ? t[0].I : i == 1 ? t[1].I : t[2].I;
+      }
+      FFP x;
+      float beta = 0.f;
+      if (c1) {
+        x = (k & 1) ? fb2 : fb1;
+      } else if (k < 6) {
+        const int v = i + 1 + j > 2 ? i + j - 2 : i + 1 + j;  // (i + 1 + j) mod 3
+        x = v == 0 ? f[0].p : v == 1 ? f[1].p : f[2].p;
+      } else if (j == 2) {
+        x = fbc;
+        beta = bb;
+      } else {
+        const int q = j == 0 ? i : i == 0 ? 2 : i - 1;
+        x = q == 0 ? fm[0] : q == 1 ? fm[1] : fm[2];
+        beta = q == 0 ? bm[0] : q == 1 ? bm[1] : bm[2];
+      }
+      ++evals;
+      if (__fadd_ru(dist_hi(B, S, x, beta), guard) <= __double2float_rd(h)) next();
+      else pend = true;
+    }
+    if (!__any_sync(0xffffffffu, pend)) break;
+    if (pend) {
+      D3 x, q;
+      if (c1) {
+        x = (k & 1) ? b2 : b1;
+      } else if (k < 6) {
+        const int v = i + 1 + j > 2 ? i + j - 2 : i + 1 + j;
+        x = v == 0 ? t[0].v : v == 1 ? t[1].v : t[2].v;
+      } else if (j == 2) {
+        x = (1.0 / 3.0) * (t[0].v + t[1].v + t[2].v);
+      } else {
+        const int e = j == 0 ? i : i == 0 ? 2 : i - 1;  // m_e is the middle of v_e and the next
+        x = 0.5 * ((e == 0 ? t[0].v : e == 1 ? t[1].v : t[2].v) + (e == 0 ? t[1].v : e == 1 ? t[2].v : t[0].v));
+      }
+      h = fmax(h, sqrt(tri_dist2(B.tri64, B.tri32, S, x, q)));
+      pend = false;
+      next();
+    }
   }
-  // the quadrilaterals (v_i, m_i, b, m_{i-1}) against S_i
-  const D3 m0 = 0.5 * (t[0].v + t[1].v), m1 = 0.5 * (t[1].v + t[2].v), m2 = 0.5 * (t[2].v + t[0].v),
-           bc = (1.0 / 3.0) * (t[0].v + t[1].v + t[2].v);
-  double ut = dmax;
-#pragma unroll 1
-  for (int k = 0; k < 9 && ut < best; ++k) {
-    const int i = k / 3, j = k % 3;
-    const int S = i == 0 ? t[0].I : i == 1 ? t[1].I : t[2].I;
-    D3 x = bc;
-    if (j == 0) x = i == 0 ? m0 : i == 1 ? m1 : m2;
-    else if (j == 1) x = i == 0 ? m2 : i == 1 ? m0 : m1;
-    raise_dist(B, S, x, ut, evals);
-  }
-  return fmin(ut, best);
+  return c1 ? h : fmin(h, best);
 }
 
 // Squared max over T of d(., {a, b}), attained at a vertex of T or where an edge of T crosses
@@ -504,32 +582,38 @@ __device__ inline double ub_u4(const VI t[3], double cap) {
   return sqrt(h2);
 }
 
-// UpperBound(T, l) of Section 4; own[i] = d(v_i, S_i).  With `full`, every bound is evaluated
-// in full (a discarded T then returns the deciding bound's own value).
+// UpperBound(T, l) of Section 4; own[i] = d(v_i, S_i).  Must be called by all 32 lanes of the
+// warp (ub_u3 votes); lanes with on == false return +inf.  With `full`, every bound is
+// evaluated in full (a discarded T then returns the deciding bound's own value).
 __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const double own[3], double l,
-                                       const uint8_t* order, int nb, bool full, int& code, unsigned& evals) {
-  if (t[0].I == t[1].I && t[1].I == t[2].I) {
-    code = 0;
-    return ub_exact(t);
-  }
+                                       const uint8_t* order, int nb, bool full, bool on, int& code, unsigned& evals) {
   double U = INFINITY;
+  code = 5;
+  if (on && t[0].I == t[1].I && t[1].I == t[2].I) {
+    code = 0;
+    U = ub_exact(t);
+    on = false;
+  }
   const EdgesD E(t);
   for (int k = 0; k < nb; ++k) {
-    double u;
+    double u = INFINITY;
     const double cap = full ? INFINITY : U;
-    switch (order[k]) {
-      case 1: u = ub_u1(t, E); break;
-      case 2: u = ub_u2(t, E, cap); break;
-      case 3: u = ub_u3(B, t, own, cap, evals); break;
-      default: u = ub_u4(t, cap); break;
+    if (order[k] == 3) {
+      const double u3 = ub_u3(B, t, own, cap, on, evals);
+      if (on) u = u3;
+    } else if (on) {
+      u = order[k] == 1 ? ub_u1(t, E) : order[k] == 2 ? ub_u2(t, E, cap) : ub_u4(t, cap);
     }
-    if (u < l) {
-      code = order[k];
-      return u;
+    if (on) {
+      if (u < l) {
+        code = order[k];
+        U = u;
+        on = false;
+      } else {
+        U = fmin(U, u);
+      }
     }
-    U = fmin(U, u);
   }
-  code = 5;
   return U;
 }
 
@@ -677,23 +761,11 @@ struct PolicyD {
     m.tri = -2;
     m.hint = a.tri;
   }
-  // The FP32 filter of the UpperBound kernels.  An item's vertices as float pairs, their
-  // distances rounded up:
+  // The FP32 filter of the UpperBound kernels.  An item's vertices for its bounds:
   __device__ static void vertices_m(const Vtx& a, const Vtx& b, const Vtx& c, VM t[3]) {
-    auto one = [](const Vtx& v) {
-      VM m;
-      m.p.h = {__double2float_rn(v.x), __double2float_rn(v.y), __double2float_rn(v.z)};
-      m.p.l = {__double2float_rn(v.x - (double)m.p.h.x), __double2float_rn(v.y - (double)m.p.h.y),
-               __double2float_rn(v.z - (double)m.p.h.z)};
-      m.dhi = __double2float_ru(v.d);
-      m.I = v.tri;
-      m.q = {0.f, 0.f, 0.f};
-      m.qerr = 0.f;
-      return m;
-    };
-    t[0] = one(a);
-    t[1] = one(b);
-    t[2] = one(c);
+    t[0] = vertex_m({a.x, a.y, a.z}, a.d, a.tri);
+    t[1] = vertex_m({b.x, b.y, b.z}, b.d, b.tri);
+    t[2] = vertex_m({c.x, c.y, c.z}, c.d, c.tri);
   }
   // An FP32 bound below this discards the item, as the FP64 bound then also does (it lies
   // below the FP32 bound up to its own rounding): l less 2^-14 of it, the slack, the distance
@@ -783,8 +855,10 @@ struct PolicyD {
     code = kDeferU4;
     return INFINITY;
   }
-  // The pass over the items left: the whole cascade in FP64, clamped to what U holds.
-  __device__ static void bound_deferred(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, double l, UT,
+  // The pass over the items left: the whole cascade in FP64, clamped to what U holds.  Must be
+  // called by all 32 lanes of the warp; only those with on == true have an item.
+  static constexpr bool kPassVotes = true;
+  __device__ static void bound_deferred(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, bool on, double l, UT,
                                         const RunParams& rp, UT& U, int& code, Counters& cnt) {
     const VI t[3] = {{{a.x, a.y, a.z}, a.d, a.tri, {a.qx, a.qy, a.qz}},
                      {{b.x, b.y, b.z}, b.d, b.tri, {b.qx, b.qy, b.qz}},
@@ -792,7 +866,7 @@ struct PolicyD {
     const double own[3] = {a.d, b.d, c.d};
     // slack is 0 in a pure FP64 run; in the certification phase of a MIXED run it is the
     // margin that covers the double rounding
-    const double u = upper_bound_d(B, t, own, l - rp.slack, rp.order, rp.n_bounds, false, code, cnt.evals) + rp.slack;
+    const double u = upper_bound_d(B, t, own, l - rp.slack, rp.order, rp.n_bounds, false, on, code, cnt.evals) + rp.slack;
     U = fmin(U, u);
   }
 };

@@ -551,7 +551,8 @@ struct PolicyM {
   __device__ static float ut_down(double x) { return __double2float_rd(x); }
   // the pass over the items left: u4, Eq. (bound_u4), for one item (certified FP32), plus the
   // slack; U holds the item's bound so far.
-  __device__ static void bound_deferred(const BvhDev&, const Vtx& a, const Vtx& b, const Vtx& c, double, float lo,
+  static constexpr bool kPassVotes = false;
+  __device__ static void bound_deferred(const BvhDev&, const Vtx& a, const Vtx& b, const Vtx& c, bool, double, float lo,
                                         const RunParams& rp, float& U, int& code, Counters&) {
     const VM t[3] = {{pos(a), a.dhi, a.tri, {a.qx, a.qy, a.qz}, a.qerr},
                      {pos(b), b.dhi, b.tri, {b.qx, b.qy, b.qz}, b.qerr},
