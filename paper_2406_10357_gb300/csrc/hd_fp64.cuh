@@ -40,8 +40,10 @@ struct NearestD {
   FFP P;               // p as a float pair
   float guard = 0.f;   // what the float forms of p and B and the FP64 test's own rounding can hide
   float pmax = 0.f;
-  // best2 rounded down / up to float, and its square root rounded up
-  float r2lo = INFINITY, r2hi = INFINITY, rhi = INFINITY;
+  // The smallest squared distance so far lies in [r2lo, r2hi], its root in [rlo, rhi]: best2
+  // rounded outward, or while candidates wait for their FP64 tests (traverse) what their FP32
+  // bounds give.
+  float r2lo = INFINITY, r2hi = INFINITY, rlo = INFINITY, rhi = INFINITY;
 
   __device__ void start(const BvhDev& B, double x, double y, double z) {
     p = {x, y, z};
@@ -65,6 +67,7 @@ struct NearestD {
   __device__ void set_radius() {
     r2lo = __double2float_rd(best2);
     r2hi = __double2float_ru(best2);
+    rlo = sqrt_dn(r2lo);
     rhi = sqrt_up(r2hi);
   }
   __device__ float coop_r2() const { return r2hi; }
@@ -76,6 +79,15 @@ struct NearestD {
     const float lo = pt_lo(P, __ldg(t), __ldg(t + 1), __ldg(t + 2), M);
     return !(__fsub_rd(lo, __fmaf_ru(0x1p-40f, __fadd_ru(pmax, M), guard)) > r);
   }
+  // Triangle j's FP32 bounds on the distance its FP64 test would compute.
+  __device__ void bounds(int j, float& lo, float& hi) const {
+    const float4* t = tri32 + 3 * (size_t)j;
+    float M;
+    lo = pt_lo(P, __ldg(t), __ldg(t + 1), __ldg(t + 2), M, &hi);
+    const float g = __fmaf_ru(0x1p-40f, __fadd_ru(pmax, M), guard);
+    lo = __fsub_rd(lo, g);
+    hi = __fadd_ru(hi, g);
+  }
   __device__ void test1(int j) {
     D3 x;
     const double d2 = tri_dist2(tri64, tri32, j, p, x);
@@ -83,7 +95,6 @@ struct NearestD {
       best2 = d2;
       best = j;
       q = x;
-      set_radius();
     }
   }
   // A leaf range in the cooperative traversal; r2 is the warp's squared radius.
@@ -91,7 +102,10 @@ struct NearestD {
     const float r = sqrt_up(r2);
     for (int j = first; j < first + count; ++j) {
       ++evals;
-      if (may(j, fminf(r, rhi))) test1(j);
+      if (may(j, fminf(r, rhi))) {
+        test1(j);
+        set_radius();
+      }
     }
   }
 };
@@ -102,20 +116,24 @@ struct NearestD {
 // lanes of the warp; inactive lanes start finished.  `first` (or -1) is a triangle to test
 // before the traversal.
 //
-// The lanes go in three steps, so that each kind of work runs on as many of them as
-// possible: a lane expands nodes until it has a leaf triangle pending; the lanes that have
-// one filter it in FP32; a lane whose triangle passes waits, and once every lane waits or is
-// finished they run the FP64 test together.  (Tested at once, the few triangles of each lane
-// that need FP64 would each cost the whole warp a test of its own.)
+// The FP64 tests are put off: a triangle certainly nearer than all before it takes their
+// place, one certainly farther than the nearest is dropped, and one the FP32 bounds leave
+// between waits with the others (up to kWait of them).  They are tested, in their order, when a
+// decision depends on it (a box distance within the bounds on the radius, a full list) and at
+// the end.  Most queries then run one or two FP64 tests instead of one for every improvement,
+// and all lanes of a warp run theirs together: a lane expands nodes until it has a leaf
+// triangle, the lanes that have one bound it in FP32, and a lane that needs a test waits until
+// every lane does or is finished.
 //
 // Bound by the FP64 pipe (2 lanes per clock and SM) before the filters: every node cost four
 // FP64 box distances, every leaf triangle an FP64 test.  Round 0 and one round of the torus
-// pair (200,000 vs 50,176 triangles, 203,860 queries): 2.20 -> 0.72 ms; 40,001 points through
-// the torus's volume (two thirds finished by warps): 3.49 -> 1.24 ms.
+// pair (200,000 vs 50,176 triangles, 203,860 queries): 2.20 ms in FP64 alone, 0.67 ms with an
+// FP64 test for each triangle that may be nearer than the best so far, 0.47 ms so.
 //
 // Returns kTravOver once more than `budget` triangles have been tested, and kTravCut once the
 // squared radius is below t.cut2 (cut_radius), with the traversal unfinished (t then holds
 // the best triangle found so far); kTravDone when it finished.
+constexpr int kWait = 4;
 constexpr int kTravDone = 0, kTravOver = 1, kTravCut = 2;
 template <bool kCut>
 __device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool active, int first, int budget) {
@@ -126,25 +144,48 @@ __device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool a
   int leaf_node = 0, slots = 0, n_slots = 0;  // leaf children waiting: their slots in leaf_node, 2 bits each
   int lfirst = 0, lcount = 0;                 // leaf triangles waiting
   bool picked = false;                        // kCut: the waiting triangle is a cut query's pick
-  int need = active ? first : -1;             // triangle waiting for its FP64 test
-  if (need >= 0) ++t.evals;
+  int wait[kWait], n_wait = 0;                // triangles waiting for their FP64 test, in order
+  bool test = false;                          // they are tested before anything else
+#pragma unroll
+  for (int q = 0; q < kWait; ++q) wait[q] = -1;
   bool done = !active;
+  if (active && first >= 0) {
+    lfirst = first;
+    lcount = 1;
+  }
   int how = kTravDone;
   const F3 plo = t.below(), phi = t.above();
+  // whether the smallest squared distance so far is below cut2 (asks for the tests where that
+  // is open)
+  const float c2lo = kCut ? __double2float_rd(t.cut2) : 0.f, c2hi = kCut ? __double2float_ru(t.cut2) : 0.f;
+  auto is_cut = [&]() {
+    if (c2hi <= t.r2lo) return false;
+    if (t.r2hi < c2lo) return true;
+    if (n_wait > 0) {
+      test = true;
+      return false;
+    }
+    return t.best2 < t.cut2;
+  };
   for (;;) {
-    while (!done && need < 0 && n_slots == 0 && lcount == 0 && !picked) {
-      bool open = false;  // node's own box distance is within rounding of the radius
+    while (!done && !test && n_slots == 0 && lcount == 0 && !picked) {
+      bool open = false;  // node's own box distance is within the bounds on the radius
       if (node < 0) {
         while (sp > 0) {
           --sp;
           const float2 e = stack_e[sp];
           if (e.x > t.r2hi) continue;
-          node = (int)stack_node[sp];
           open = !(e.y < t.r2lo);
+          if (open && n_wait > 0) {  // decided after the tests
+            ++sp;
+            test = true;
+            break;
+          }
+          node = (int)stack_node[sp];
           break;
         }
         if (node < 0) {
-          done = true;
+          done = !test;
           continue;
         }
       }
@@ -170,11 +211,12 @@ __device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool a
         continue;
       }
       if constexpr (kCut) {
-        if (t.best2 < t.cut2) {
+        if (is_cut()) {
           how = kTravCut;
           done = true;
           continue;
         }
+        if (test) continue;  // node is kept for after the tests
       }
       ++c.nodes;
       // the children's intervals; those certainly beyond the radius, and missing ones, at +inf
@@ -276,45 +318,78 @@ __device__ inline int traverse(const BvhDev& B, NearestD& t, Counters& c, bool a
       }
       node = -1;
     }
-    if (!done && need < 0) {
+    if (!done && !test) {
       if (lcount == 0) {
         if (kCut && picked) {
-          picked = false;
-          if (t.best2 < t.cut2) {
+          if (is_cut()) {
             how = kTravCut;
             done = true;
           }
+          picked = test;  // asked again after the tests
         }
-        if (!done && n_slots > 0) {
+        if (!done && !test && n_slots > 0) {
           const int s = slots & 3;
-          slots >>= 2;
-          --n_slots;
           const float* nf = reinterpret_cast<const float*>(B.nodes + leaf_node) + s;
           const float ax = __ldg(nf), ay = __ldg(nf + 4), az = __ldg(nf + 8);
           const float bx = __ldg(nf + 12), by = __ldg(nf + 16), bz = __ldg(nf + 20);
           const unsigned k = __ldg(reinterpret_cast<const unsigned*>(nf) + 24);
           bool in = box_hi2(plo, phi, ax, ay, az, bx, by, bz) < t.r2lo;
-          if (!in && !(box_lo2(plo, phi, ax, ay, az, bx, by, bz) > t.r2hi))
-            in = box_dist2(t.p, ax, ay, az, bx, by, bz) < t.best2;
+          if (!in && !(box_lo2(plo, phi, ax, ay, az, bx, by, bz) > t.r2hi)) {
+            if (n_wait > 0) test = true;
+            else in = box_dist2(t.p, ax, ay, az, bx, by, bz) < t.best2;
+          }
+          if (!test) {
+            slots >>= 2;
+            --n_slots;
+          }
           if (in) {
             lfirst = code_ref(k);
             lcount = code_count(k);
           }
         }
       }
-      if (!done && lcount > 0) {
+      if (!done && !test && lcount > 0) {
         ++t.evals;
-        if (t.may(lfirst, t.rhi)) need = lfirst;
+        float lo, hi;
+        t.bounds(lfirst, lo, hi);
+        if (hi < t.rlo) {  // certainly the nearest so far
+          t.best2 = INFINITY;
+          n_wait = 1;
+          wait[0] = lfirst;
+          t.rlo = fmaxf(lo, 0.f);
+          t.rhi = hi;
+          t.r2lo = __fmul_rd(t.rlo, t.rlo);
+          t.r2hi = __fmul_ru(hi, hi);
+        } else if (!(lo > t.rhi)) {
+#pragma unroll
+          for (int q = 0; q < kWait; ++q)
+            if (q == n_wait) wait[q] = lfirst;
+          ++n_wait;
+          t.rlo = fminf(t.rlo, fmaxf(lo, 0.f));
+          t.r2lo = fminf(t.r2lo, __fmul_rd(t.rlo, t.rlo));
+          if (hi < t.rhi) {
+            t.rhi = hi;
+            t.r2hi = __fmul_ru(hi, hi);
+          }
+          test = n_wait == kWait || !(hi < INFINITY);  // (no upper bound: its own test is needed)
+        }
         ++lfirst;
         --lcount;
       }
     }
-    if (__any_sync(0xffffffffu, !done && need < 0)) continue;
-    if (__all_sync(0xffffffffu, done)) break;
-    if (need >= 0) {
-      t.test1(need);
-      need = -1;
-    }
+    if (__any_sync(0xffffffffu, !done && !test)) continue;
+    if (!__any_sync(0xffffffffu, n_wait > 0)) break;
+    do {
+      if (n_wait > 0) {
+        t.test1(wait[0]);
+#pragma unroll
+        for (int q = 0; q + 1 < kWait; ++q) wait[q] = wait[q + 1];
+        if (--n_wait == 0) {
+          t.set_radius();
+          test = false;
+        }
+      }
+    } while (__any_sync(0xffffffffu, n_wait > 0));
   }
   return how;
 }
