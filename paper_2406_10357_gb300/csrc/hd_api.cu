@@ -506,6 +506,7 @@ int hd_upper_bounds(const hd_bvh* B, const double* T, const double* Td, const in
   rp.slack = 0.0;
   rp.slack_f = 0.f;
   rp.defer_u4 = 0;
+  rp.keep_order = 0;
   rp.parent_clamp = 0;
   memcpy(rp.order, o.order, 4);
   rp.n_bounds = o.n_bounds;

@@ -1356,6 +1356,7 @@ int run_batch(const hd_bvh* const* Bs, const hd_mesh* As, int64_t npairs, double
   rp.slack_f = 0.f;
   rp.dyn = nullptr;
   rp.defer_u4 = 1;
+  rp.keep_order = 0;
   rp.parent_clamp = (o.flags & HD_FLAG_NO_PARENT_CLAMP) ? 0 : 1;
   memcpy(rp.order, o.order, 4);
   rp.n_bounds = o.n_bounds;

@@ -836,7 +836,7 @@ __global__ void HD_BOUND_REGS k_bound_faces(BvhDev B, const typename P::Vtx* poo
     flush_tally(st, ty);
     return;
   }
-  const int lanes = spread_lanes(nFA, P::kSpreadBounds);
+  const int lanes = rp.keep_order ? 32 : spread_lanes(nFA, P::kSpreadBounds);
   for (;;) {
     const int64_t base = warp_batch(&st->b_next, lanes);
     if (base >= nFA) break;
@@ -871,7 +871,7 @@ __device__ inline void bound_u4_body(BvhDev B, const typename P::Vtx* pool, cons
   const Thresholds<P>& th = lv.th;
   Counters c;
   Tally<P> ty;
-  const int lanes = spread_lanes(n, P::kSpreadBounds), lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int lanes = rp.keep_order ? 32 : spread_lanes(n, P::kSpreadBounds), lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   for (int64_t base = (blockIdx.x * (int64_t)wpb + (threadIdx.x >> 5)) * lanes; base < n;
        base += (int64_t)gridDim.x * wpb * lanes) {
     const int64_t t = base + lane;
@@ -1076,7 +1076,7 @@ __device__ inline void bound_children_body(BvhDev B, const typename P::Vtx* pool
     flush_tally(st, ty);
     return;
   }
-  const int lanes = spread_lanes(4 * (int64_t)S, P::kSpreadBounds);
+  const int lanes = rp.keep_order ? 32 : spread_lanes(4 * (int64_t)S, P::kSpreadBounds);
   for (;;) {
     const int64_t base = warp_batch(&st->b_next, lanes);
     if (base >= 4 * (int64_t)S) break;
@@ -1934,6 +1934,7 @@ int run_bnb(const RunIO& io) {
   rp.slack_f = 0.f;
   rp.dyn = dyn;
   rp.defer_u4 = 1;
+  rp.keep_order = (o.flags & HD_FLAG_SHARE_MIDPOINTS) ? 1 : 0;
   rp.parent_clamp = (o.flags & HD_FLAG_NO_PARENT_CLAMP) ? 0 : 1;
   memcpy(rp.order, o.order, 4);
   rp.n_bounds = o.n_bounds;

@@ -239,6 +239,8 @@ struct RunParams {
   float slack_f;  // slack rounded up to float
   int defer_u4;   // a trailing u4 is evaluated in the second pass of the bounds
   int parent_clamp;  // children's U is clamped to their parent's U
+  int keep_order;    // neighbouring items stay together in the frontier (shared midpoints): no
+                     // short lists spread over more warps
   const DynParams* dyn;  // if set, eps / slack / slack_f are taken from here on the device
 };
 
