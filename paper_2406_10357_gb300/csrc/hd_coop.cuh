@@ -57,7 +57,8 @@ constexpr int kCoopMinBlocks = HD_COOP_MIN_BLOCKS;
 constexpr int kCoopMinBlocksCut = HD_COOP_MIN_BLOCKS_CUT;
 // The FP64 policy's cooperative traversal keeps doubles in flight (its query point, the best
 // squared distance and closest point, the triangle being tested): at 40 registers it spills
-// heavily, so it asks for fewer blocks per SM, and its lanes keep their queries longer.
+// heavily, so it asks for fewer blocks per SM (40,001 points in a volume with 4, 5, 6, 7, 8
+// blocks: 1.20, 1.23, 1.23, 1.29, 1.27 ms), and its lanes keep their queries longer.
 #ifndef HD_COOP_MIN_BLOCKS_D
 #define HD_COOP_MIN_BLOCKS_D 4
 #endif
