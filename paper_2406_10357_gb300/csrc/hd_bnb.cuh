@@ -1702,8 +1702,11 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
       TraceScope tr(HD_K_LONG, s);
       // The reordering where this round may hand off a list worth it: not where the last round
       // read handed off few, of a frontier at least a quarter of this one's bound.
-      if (last_long < 0 || 8 * (int64_t)last_long >= kSortMin) sort_long<P>(B, R.pool, R.longq, st, true, sms, s, rp.dyn);
-      launch_query_long<P>(cuts, B, R.pool, R.longq, st, rp.slack, rp.dyn, true, s);
+      // (Left out, the list keeps its order: the reordered copy is not this round's.)
+      LongList ll = R.longq;
+      if (last_long < 0 || 8 * (int64_t)last_long >= kSortMin) sort_long<P>(B, R.pool, ll, st, true, sms, s, rp.dyn);
+      else ll.sorted = nullptr;
+      launch_query_long<P>(cuts, B, R.pool, ll, st, rp.slack, rp.dyn, true, s);
     }
     {
       TraceScope tr(HD_K_BOUND, s);
