@@ -136,6 +136,12 @@ struct PairAcc {
   int pair;  // -1: empty
 };
 constexpr int kMaxWarps = 32;  // warps of a block
+// Batches of at least this many pairs: a warp whose items belong to more than one pair adds them
+// lane by lane instead.  There such warps hold many pairs, each a pass of the reductions, and
+// the lanes' additions spread over as many states; with fewer pairs they meet in a few and are
+// what the reductions are for.  128 pairs: 46.2 ms with reductions, 62.0 lane by lane; 512
+// pairs: 207.1 and 197.5 ms.
+constexpr int kAccDirectPairs = 256;
 
 __device__ inline void acc_reset(PairAcc& a, int pair) {
   a.l = a.uret = a.umax = 0ull;
@@ -190,10 +196,32 @@ __device__ inline unsigned long long group_max(unsigned g, float v) {
 // nothing to add); `a` is the warp's accumulator.  l stays non-negative (a certified vertex
 // distance less its slack can be below 0), which the maximum on its bits needs.
 template <class P>
-__device__ inline void acc_batch(PairAcc& a, RunState* sts, int pair, const PairDelta<P>& d, bool long_pass = false) {
+__device__ inline void acc_batch(PairAcc& a, const BatchCtx& x, int pair, const PairDelta<P>& d, bool long_pass = false) {
+  RunState* sts = x.sts;
   const int lane = threadIdx.x & 31;
   if (d.c.err && pair >= 0) atomicExch(&sts[pair].err, 1);
   unsigned left = __ballot_sync(0xffffffffu, pair >= 0);
+  if (x.npairs >= kAccDirectPairs && warp_pair(pair) == -2) {
+    if (pair >= 0) {
+      PairAcc b;
+      acc_reset(b, pair);
+      b.evals = d.c.evals;
+      b.leaf = d.c.leaf;
+      b.boxes = d.c.boxes;
+      b.nodes = d.c.nodes;
+      b.escalations = d.c.escalations;
+      b.nq = (unsigned)d.nq;
+      if (d.nq) b.l = (unsigned long long)__double_as_longlong(fmax(d.l, 0.0));
+#pragma unroll
+      for (int k = 0; k < 6; ++k) b.discards[k] = d.discard == k;
+      b.retired = (unsigned)d.retired;
+      b.kept = (unsigned)d.kept;
+      b.uret = (unsigned long long)__double_as_longlong(fmax((double)d.uret, 0.0));
+      b.umax = (unsigned long long)__double_as_longlong(fmax((double)d.umax, 0.0));
+      acc_apply(sts, b, long_pass);
+    }
+    return;
+  }
   while (left) {  // one pair of the warp at a time (uniform)
     const int p = __shfl_sync(0xffffffffu, pair, __ffs(left) - 1);
     const unsigned g = __ballot_sync(0xffffffffu, pair == p);
@@ -439,7 +467,7 @@ __global__ void HD_QUERY_REGS k_batch_query(BatchCtx x, typename P::Vtx* pool, c
         d.nq = 1;
       }
     }
-    acc_batch(acc, x.sts, q ? p : -1, d);
+    acc_batch(acc, x, q ? p : -1, d);
   }
   acc_end(acc, x.sts);
 }
@@ -473,7 +501,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, P::kCoopBlocks)
       d.l = P::lower(v) - x.dyn[p].slack;
       d.nq = 1;
     }
-    acc_batch(acc, x.sts, p, d, true);
+    acc_batch(acc, x, p, d, true);
   }
   acc_end(acc, x.sts, true);
 }
@@ -530,7 +558,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
             classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
           }
         }
-        acc_batch(acc, x.sts, need ? -1 : p, ty);
+        acc_batch(acc, x, need ? -1 : p, ty);
         const unsigned m = __ballot_sync(0xffffffffu, need);
         if (need) q[qn + __popc(m & lt)] = e;
         qn += __popc(m);
@@ -558,7 +586,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
       }
       qn -= take;
       __syncwarp();  // the entries taken are read before new ones overwrite them
-      acc_batch(acc, x.sts, p, ty);
+      acc_batch(acc, x, p, ty);
     }
   }
   acc_end(acc, x.sts);
@@ -634,7 +662,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
       it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, ty.c);
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    acc_batch(acc, x.sts, p, ty);
+    acc_batch(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }
@@ -669,7 +697,7 @@ __global__ void k_batch_bound_u4(BatchCtx x, const typename P::Vtx* pool, const 
       if (on) classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, nullptr, nullptr, ty);
       else p = -1;
     }
-    acc_batch(acc, x.sts, p, ty);
+    acc_batch(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }
@@ -772,7 +800,7 @@ __global__ void k_batch_select(BatchCtx x, const typename P::Item* front, const 
         }
       }
     }
-    acc_batch(acc, x.sts, p, ty);
+    acc_batch(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }
@@ -838,7 +866,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
       if (pl.rp.parent_clamp && Up < it.U) it.U = Up;
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    acc_batch(acc, x.sts, p, ty);
+    acc_batch(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }

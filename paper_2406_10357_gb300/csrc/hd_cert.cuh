@@ -197,8 +197,11 @@ __device__ inline float box_hi2(F3 plo, F3 phi, float lx, float ly, float lz, fl
 // the largest local coordinate.  Non-finite arithmetic ends in 0.
 // With `hi`, also an upper bound (the length of the point found plus the 48 u M margin of
 // pt_cert), or +inf for an ill-conditioned triangle (the classification's own threshold):
-// there a closest point computed in FP64 can be farther than the true one.
-__device__ inline float pt_lo(const FFP& P, float4 a4, float4 b4, float4 c4, float& M, float* hi = nullptr) {
+// there a closest point computed in FP64 can be farther than the true one.  The triangle B was
+// given may be ill-conditioned where its float form is not, so +inf too unless eta is far
+// below the edges (the threshold leaves a height of 4e-3 of the shorter edge).
+__device__ inline float pt_lo(const FFP& P, float4 a4, float4 b4, float4 c4, float& M, float* hi = nullptr,
+                              float eta = 0.f) {
   const F3 A = local_off(a4, P), B = local_off(b4, P), C = local_off(c4, P);
   M = fmaxf(fmaxf(amax3(A), amax3(B)), fmaxf(amax3(C), amax3(P.l)));
   float v, w;
@@ -207,7 +210,8 @@ __device__ inline float pt_lo(const FFP& P, float4 a4, float4 b4, float4 c4, flo
   const F3 Q = {fmaf(w, E2.x, fmaf(v, E1.x, A.x)), fmaf(w, E2.y, fmaf(v, E1.y, A.y)), fmaf(w, E2.z, fmaf(v, E1.z, A.z))};
   if (hi) {
     const float aa = dotf(E1, E1), cc = dotf(E2, E2), bc = dotf(E1, E2);
-    *hi = aa * cc - bc * bc > 2e-5f * aa * cc ? __fadd_ru(norm_ru(Q), __fmul_ru(48.f * kU, M)) : INFINITY;
+    const bool sound = aa * cc - bc * bc > 2e-5f * aa * cc && eta * eta <= 1e-6f * fminf(aa, cc);
+    *hi = sound ? __fadd_ru(norm_ru(Q), __fmul_ru(48.f * kU, M)) : INFINITY;
   }
   F3 n = Q;  // vertex region
   if (region == 0) {  // face: the plane normal

@@ -83,7 +83,7 @@ struct NearestD {
   __device__ void bounds(int j, float& lo, float& hi) const {
     const float4* t = tri32 + 3 * (size_t)j;
     float M;
-    lo = pt_lo(P, __ldg(t), __ldg(t + 1), __ldg(t + 2), M, &hi);
+    lo = pt_lo(P, __ldg(t), __ldg(t + 1), __ldg(t + 2), M, &hi, guard);  // (guard: eta and 1e-37)
     const float g = __fmaf_ru(0x1p-40f, __fadd_ru(pmax, M), guard);
     lo = __fsub_rd(lo, g);
     hi = __fadd_ru(hi, g);

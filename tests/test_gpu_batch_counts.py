@@ -27,11 +27,12 @@ def hd():
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 @pytest.mark.parametrize("order", [(1, 2, 3, 4), (3, 2)])
-def test_counts_of_tiny_pairs_equal_single_runs(hd, precision, order):
+@pytest.mark.parametrize("n_pairs", [75, 300])  # sums by reductions, and lane by lane (from 256 pairs)
+def test_counts_of_tiny_pairs_equal_single_runs(hd, precision, order, n_pairs):
     rng = np.random.default_rng(3)
     VB, FB, _ = mg.torus(1.0, 0.3, 14, 7)
     pairs = []
-    for i in range(75):  # 1 to 9 faces each, so 32 items span several pairs
+    for i in range(n_pairs):  # 1 to 9 faces each, so 32 items span several pairs
         n = 1 + i % 9
         c = VB[rng.integers(len(VB), size=n)]
         V = (c[:, None] + rng.normal(0, 0.15, (n, 3, 3))).reshape(-1, 3)
