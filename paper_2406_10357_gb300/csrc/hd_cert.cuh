@@ -297,6 +297,41 @@ __device__ inline float ubm_u2(const VM t[3], const EdgesM& E) {
   return __fadd_ru(g, fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi)));
 }
 
+// Lower bound of u2 for every g its acute test may choose: g is at least half the longest edge,
+// and the circumradius (rounded down) where T is certainly acute.  0 where an edge leaves the
+// float range.
+__device__ inline float ubm_u2_lo(const VM t[3], const EdgesM& E) {
+  float lo[3];  // norm_ru is within 2^-18 above the length, or 1e-15 of it (sqrt_up)
+#pragma unroll
+  for (int i = 0; i < 3; ++i) lo[i] = fmaxf(__fsub_rd(__fmul_rd(E.hi[i], 1.f - 0x1p-18f), 2e-15f), 0.f);
+  const float hk = fmaxf(E.hi[0], fmaxf(E.hi[1], E.hi[2]));
+  if (!(hk < INFINITY)) return 0.f;
+  float g = 0.5f * fmaxf(lo[0], fmaxf(lo[1], lo[2]));
+  if (__fmaf_rd(lo[0], lo[0], __fmaf_rd(lo[1], lo[1], __fmul_rd(lo[2], lo[2]))) > __fmul_ru(__fmul_ru(2.f, hk), hk)) {
+    const F3 a = E.e[2], b = {-E.e[1].x, -E.e[1].y, -E.e[1].z};
+    const F3 cr = {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+    const float c2 = __fadd_ru(norm_ru(cr), __fmul_ru(__fmul_ru(32.f * kU, amax3(a)), amax3(b)));  // 2|T|, rounded up
+    g = fmaxf(g, div_dn(__fmul_rd(__fmul_rd(lo[0], lo[1]), lo[2]), __fmul_ru(2.f, c2)));
+  }
+  return __fadd_rd(g, __fmul_rd(fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi)), 1.f - 0x1p-20f));
+}
+
+// Lower bound of u4 whichever edge of T is taken for the shortest: H(q_i, q_j) is at least the
+// distance from the third vertex to the nearer of q_i and q_j.  The distances are plain float,
+// within 16 u M of the exact ones (M: the largest coordinate relative to T's first vertex).
+__device__ inline float ubm_u4_lo(const VM t[3]) {
+  const F3 x[3] = {f3(0.f, 0.f, 0.f), edge(t[0], t[1]), edge(t[0], t[2])};
+  const F3 q[3] = {t[0].q, x[1] + t[1].q, x[2] + t[2].q};
+  float d2 = INFINITY;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const F3 a = x[i] - q[(i + 1) % 3], b = x[i] - q[(i + 2) % 3];
+    d2 = fminf(d2, fminf(dotf(a, a), dotf(b, b)));
+  }
+  const float M = fmaxf(fmaxf(amax3(x[1]), amax3(x[2])), fmaxf(amax3(t[0].q), fmaxf(amax3(t[1].q), amax3(t[2].q))));
+  return __fsub_rd(sqrt_dn(d2), __fmul_ru(0x1p-18f, M));
+}
+
 // Upper bound of d(x, S) for the float triangle S = (a4, b4, c4), x = h + l, computed without
 // branches: the distance to the projection of x onto the plane of S when it falls inside S
 // (well-conditioned triangles only), else to the nearest of the three edge projections.  Any

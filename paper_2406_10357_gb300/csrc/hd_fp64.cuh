@@ -836,19 +836,39 @@ struct PolicyD {
     m.tri = -2;
     m.hint = a.tri;
   }
-  // The FP32 filter of the UpperBound kernels.  An item's vertices for its bounds:
+  // The FP32 filter of the UpperBound kernels.  An item's vertices for its bounds (q only for
+  // ubm_u4_lo):
   __device__ static void vertices_m(const Vtx& a, const Vtx& b, const Vtx& c, VM t[3]) {
     t[0] = vertex_m({a.x, a.y, a.z}, a.d, a.tri);
     t[1] = vertex_m({b.x, b.y, b.z}, b.d, b.tri);
     t[2] = vertex_m({c.x, c.y, c.z}, c.d, c.tri);
   }
-  // An FP32 bound below this discards the item, as the FP64 bound then also does (it lies
-  // below the FP32 bound up to its own rounding): l less 2^-14 of it, the slack, the distance
-  // of B's float vertices from its own, and the float pairs' rounding.
-  __device__ static float filter_limit(const BvhDev& B, const VM t[3], float lf, const RunParams& rp) {
+  __device__ static F3 foot_m(const Vtx& v) {
+    return {__double2float_rn(v.qx - v.x), __double2float_rn(v.qy - v.y), __double2float_rn(v.qz - v.z)};
+  }
+  // What the filter compares with: an FP32 upper bound below u12 (u1, u2) or u3 discards the
+  // item, as the FP64 bound then also does (it lies below the FP32 bound up to its own rounding):
+  // l less 2^-14 of it, the slack, the float pairs' rounding (u1 and u2 move by no more than the
+  // vertices do: g is the radius of T's smallest enclosing circle) and, for u3, the distance
+  // of B's float vertices from its own.  An FP32 lower bound of at least `keep` shows that the FP64
+  // bound does not discard it (2e-15: what sqrt_up adds to tiny lengths).  Between the two the
+  // item is left to the FP64 cascade, so that the bound a discard is counted for is the one
+  // FP64 alone finds.
+  struct Limits {
+    float u12, u3, keep;
+  };
+  __device__ static Limits limits(const BvhDev& B, const VM t[3], float lf, const RunParams& rp) {
     const float pmax = fmaxf(amax3(t[0].p.h), fmaxf(amax3(t[1].p.h), amax3(t[2].p.h)));
-    const float guard = __fadd_ru(__fmaf_ru(0x1p-38f, pmax, __fadd_ru(__ldg(B.meta), 1e-37f)), rp.slack_f);
-    return __fsub_rd(__fmul_rd(lf, 1.f - 0x1p-14f), guard);
+    const float rep = __fadd_ru(__fmaf_ru(0x1p-38f, pmax, 1e-37f), rp.slack_f);
+    Limits m;
+    m.u12 = __fsub_rd(__fmul_rd(lf, 1.f - 0x1p-14f), rep);
+    m.u3 = __fsub_rd(m.u12, __ldg(B.meta));
+    m.keep = __fadd_ru(__fmaf_ru(lf, 1.f + 0x1p-13f, rep), 2e-15f);
+    return m;
+  }
+  // u1 or u2 (u: upper bound, lo: lower bound) decides: 1 discards, 0 does not, -1 is left open
+  __device__ static int verdict(const Limits& m, float u, float lo) {
+    return u < m.u12 ? 1 : lo >= m.keep && lo < INFINITY ? 0 : -1;
   }
   // The cascade's part in the UpperBound kernels: the exact case, and the items that certified
   // FP32 bounds u1..u3 discard.  Every other item is left (kDeferU4, U = +inf) to the pass
@@ -873,28 +893,29 @@ struct PolicyD {
     }
     VM t[3];
     vertices_m(a, b, c, t);
-    const float lim = filter_limit(B, t, lf, rp);
+    const Limits m = limits(B, t, lf, rp);
     const EdgesM E(t);
-    const float u1 = ubm_u1(t, E);
-    if (u1 < lim) {
-      *code = 1;
-      *U = (UT)u1;
-      return false;
-    }
-    const float u2 = ubm_u2(t, E);
-    if (u2 < lim) {
+    const float u1 = ubm_u1(t, E), u2 = ubm_u2(t, E);
+    int v = verdict(m, u1, u1);
+    *code = 1;
+    *U = (UT)u1;
+    if (v == 0) {
+      v = verdict(m, u2, ubm_u2_lo(t, E));
       *code = 2;
       *U = (UT)u2;
-      return false;
+    }
+    if (v < 0) {
+      *code = kDeferU4;
+      *U = INFINITY;
     }
     *u12 = fminf(u1, u2);
-    return true;
+    return v == 0;
   }
   __device__ static UT paper_u3(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf, const RunParams& rp,
                                 float, float, int& code, Counters& cnt) {
     VM t[3];
     vertices_m(a, b, c, t);
-    const float lim = filter_limit(B, t, lf, rp);
+    const float lim = limits(B, t, lf, rp).u3;
     if (lim > 0.f) {
       const float u3 = ubm_u3<true>(B, t, lim, cnt.evals);
       if (u3 < lim) {
@@ -914,20 +935,35 @@ struct PolicyD {
     }
     VM t[3];
     vertices_m(a, b, c, t);
-    const float lim = filter_limit(B, t, lf, rp);
-    if (lim > 0.f) {
-      const EdgesM E(t);
-      for (int k = 0; k < rp.n_bounds; ++k) {
-        const int o = rp.order[k];
-        if (o == 4) continue;
-        const float u = o == 1 ? ubm_u1(t, E) : o == 2 ? ubm_u2(t, E) : ubm_u3<true>(B, t, lim, cnt.evals);
-        if (u < lim) {
-          code = o;
-          return (UT)u;
-        }
+    const Limits m = limits(B, t, lf, rp);
+    code = kDeferU4;
+    if (!(m.u12 > 0.f)) return INFINITY;
+    const EdgesM E(t);
+    for (int k = 0; k < rp.n_bounds; ++k) {
+      const int o = rp.order[k];
+      float u = INFINITY;
+      int v;
+      if (o == 1) {
+        u = ubm_u1(t, E);
+        v = verdict(m, u, u);
+      } else if (o == 2) {
+        u = ubm_u2(t, E);
+        v = verdict(m, u, ubm_u2_lo(t, E));
+      } else if (o == 3) {
+        if (m.u3 > 0.f) u = ubm_u3<true>(B, t, m.u3, cnt.evals);
+        v = u < m.u3 ? 1 : -1;
+      } else {
+        t[0].q = foot_m(a);
+        t[1].q = foot_m(b);
+        t[2].q = foot_m(c);
+        v = verdict(m, INFINITY, ubm_u4_lo(t));
+      }
+      if (v < 0) break;
+      if (v == 1) {
+        code = o;
+        return (UT)u;
       }
     }
-    code = kDeferU4;
     return INFINITY;
   }
   // The pass over the items left: the whole cascade in FP64, clamped to what U holds.  Must be
