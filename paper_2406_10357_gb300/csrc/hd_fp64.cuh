@@ -657,11 +657,13 @@ __device__ inline double ub_u4(const VI t[3], double cap) {
   return sqrt(h2);
 }
 
-// UpperBound(T, l) of Section 4; own[i] = d(v_i, S_i).  Must be called by all 32 lanes of the
-// warp (ub_u3 votes); lanes with on == false return +inf.  With `full`, every bound is
-// evaluated in full (a discarded T then returns the deciding bound's own value).
-__device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const double own[3], double l,
-                                       const uint8_t* order, int nb, bool full, bool on, int& code, unsigned& evals) {
+// UpperBound(T, l) of Section 4; own(i) = d(v_i, S_i), asked for only where u3 is reached.  Must
+// be called by all 32 lanes of the warp (ub_u3 votes); lanes with on == false return +inf.
+// With `full`, every bound is evaluated in full (a discarded T then returns the deciding bound's
+// own value).
+template <class Own>
+__device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const Own& own, double l, const uint8_t* order,
+                                       int nb, bool full, bool on, int& code, unsigned& evals) {
   double U = INFINITY;
   code = 5;
   if (on && t[0].I == t[1].I && t[1].I == t[2].I) {
@@ -674,7 +676,12 @@ __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const dou
     double u = INFINITY;
     const double cap = full ? INFINITY : U;
     if (order[k] == 3) {
-      const double u3 = ub_u3(B, t, own, cap, on, evals);
+      double d[3] = {0.0, 0.0, 0.0};
+      if (on) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) d[i] = own(i);
+      }
+      const double u3 = ub_u3(B, t, d, cap, on, evals);
       if (on) u = u3;
     } else if (on) {
       u = order[k] == 1 ? ub_u1(t, E) : order[k] == 2 ? ub_u2(t, E, cap) : ub_u4(t, cap);
@@ -974,7 +981,7 @@ struct PolicyD {
     const VI t[3] = {{{a.x, a.y, a.z}, a.d, a.tri, {a.qx, a.qy, a.qz}},
                      {{b.x, b.y, b.z}, b.d, b.tri, {b.qx, b.qy, b.qz}},
                      {{c.x, c.y, c.z}, c.d, c.tri, {c.qx, c.qy, c.qz}}};
-    const double own[3] = {a.d, b.d, c.d};
+    auto own = [&](int i) { return t[i].d; };
     // slack is 0 in a pure FP64 run; in the certification phase of a MIXED run it is the
     // margin that covers the double rounding
     const double u = upper_bound_d(B, t, own, l - rp.slack, rp.order, rp.n_bounds, false, on, code, cnt.evals) + rp.slack;
