@@ -544,39 +544,44 @@ __global__ void k_long_hist(BvhDev B, const typename P::Vtx* pool, LongList ll, 
     atomicAdd(&ll.buckets[long_cell<P>(B, pool[ll.idx[i]], st, dyn)], 1u);
 }
 
-// Exclusive scan of the cell counts: one block of 1024 threads, kSortBuckets / 1024 rows of
-// 1024 consecutive counters, each row scanned across the block (coalesced) and carried on.
+// Exclusive scan of the cell counts: one block of 1024 threads, each warp a run of 1024
+// consecutive counters, all loaded first (coalesced) and scanned in registers, so that only the
+// warps' totals wait at a barrier.  (Row after row across the block, with four barriers
+// each, it took 14 us of the 16 it added to a call of hd_nearest.)
 __device__ inline void scan_buckets(unsigned* buckets) {
-  constexpr int kRows = kSortBuckets / 1024;
+  constexpr int kPer = kSortBuckets / (4 * 1024);
+  static_assert(4 * 1024 * kPer == kSortBuckets, "whole rows");
   __shared__ unsigned wtot[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  unsigned val[kRows];  // every row's counter first: the loads overlap instead of one per row
-#pragma unroll
-  for (int row = 0; row < kRows; ++row) val[row] = buckets[row * 1024 + threadIdx.x];
-  unsigned carry = 0;
-#pragma unroll
-  for (int row = 0; row < kRows; ++row) {
-    const int i = row * 1024 + threadIdx.x;
-    const unsigned v = val[row];
-    unsigned x = v;  // inclusive warp scan
+  uint4* row = reinterpret_cast<uint4*>(buckets) + 32 * kPer * w + lane;
+  auto scan = [lane](unsigned x) {
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
     }
-    if (lane == 31) wtot[w] = x;
-    __syncthreads();
-    if (w == 0) {  // the warps' totals, scanned
-      unsigned t = wtot[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      wtot[lane] = t;
-    }
-    __syncthreads();
-    buckets[i] = carry + (w ? wtot[w - 1] : 0u) + x - v;
-    carry += wtot[31];
-    __syncthreads();  // wtot is written again by the next row
+    return x;
+  };
+  uint4 v[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) v[k] = __ldcg(row + 32 * k);
+  unsigned at[kPer], carry = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const unsigned sum = v[k].x + v[k].y + v[k].z + v[k].w, x = scan(sum);
+    at[k] = carry + x - sum;
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) wtot[w] = carry;
+  __syncthreads();
+  const unsigned t = wtot[lane], base = __shfl_sync(0xffffffffu, scan(t) - t, w);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    uint4 o;
+    o.x = base + at[k];
+    o.y = o.x + v[k].x;
+    o.z = o.y + v[k].y;
+    o.w = o.z + v[k].z;
+    row[32 * k] = o;
   }
 }
 
@@ -2040,26 +2045,49 @@ int run_bnb(const RunIO& io) {
 
 // The order external points are queried in.  Points that follow each other in space share
 // nodes and branches in a warp; points in random order share neither.  So a large set is
-// grouped by Morton cell of B's box (a counting sort: k_points_cell, k_points_scan,
-// k_points_place), unless its own order is coherent already, that is, unless few neighbours
-// lie in different cells; the results go back in the caller's order, and each query's result
-// does not depend on its place.  500,000 random points near a torus of 50,176 triangles,
-// MIXED: 0.724 -> 0.661 ms per call, the sort included.  Below kPointSortMin points the
-// queries are bound by their latency and the sort does not pay.
+// grouped by Morton cell of B's box (a counting sort: k_points_cell counts, k_points_in places),
+// unless its own order is coherent already, that is, unless more than a quarter of neighbours
+// lie in cells that do not touch; the results go back in the caller's order, and each query's
+// result does not depend on its place.  Either way the queries handed off come in a useful order
+// too, and their own reordering (sort_long, three launches) is left out, which pays for the
+// kernel that counts.  Points near a torus of 50,176 triangles, MIXED, us, without any of this /
+// with it (in scan order, at random within 0.003 of it, at random within 0.03):
+//    32,768 points   81 /  84    87 /  90   131 / 129
+//   131,072 points  154 / 132   181 / 143   251 / 224
+//   500,000 points  338 / 341   444 / 372   674 / 601
+// and 64,000 in a grid through its volume 664 / 453.  Below 32,768 the queries are bound by their
+// latency: the kernel more is 4 of 76 us there and brings nothing.
 struct PointOrder {
   int* place = nullptr;  // record of each point (null: the points' own order)
   int* cell = nullptr;
   unsigned* buckets = nullptr;  // kSortBuckets counters, zero at the start
-  unsigned* jumps = nullptr;    // neighbouring points in different cells, zero at the start
+  // blocks of k_points_cell that are through << 32 | neighbouring points in cells that do not
+  // touch; zero at the start
+  unsigned long long* tally = nullptr;
 };
 constexpr int64_t kPointSortMin = 1 << 15;
+constexpr int kPointCellBlock = 1024;  // scan_buckets' block
 
 __device__ inline bool points_sorted(const PointOrder& o, int64_t n) {
-  return o.place && (int64_t)*o.jumps * 4 > n;
+  return o.place && (int64_t)(unsigned)*o.tally * 4 > n;
 }
 
+// Whether cells a and b are the same or neighbours, diagonally too (Morton codes: an axis's
+// difference, taken in place on its bits, is 0, 1 or -1).
+__device__ inline bool cells_touch(int a, int b) {
+  bool near = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int m = 0x1249 << k, d = ((a & m) - (b & m)) & m;
+    near &= d == 0 || d == 1 << k || d == m;
+  }
+  return near;
+}
+
+// The cell of every point, the points per cell and the jumps; the last block through turns the
+// counts into each cell's first place, where the order is not coherent.
 template <typename T>
-__global__ void k_points_cell(BvhDev B, const T* P_, int64_t n, PointOrder o) {
+__global__ void __launch_bounds__(kPointCellBlock) k_points_cell(BvhDev B, const T* P_, int64_t n, PointOrder o) {
   grid_dep_wait();
   grid_dep_launch();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -2067,27 +2095,23 @@ __global__ void k_points_cell(BvhDev B, const T* P_, int64_t n, PointOrder o) {
   const bool on = i < n;
   const int c = on ? (int)long_bucket(B, (float)P_[3 * i], (float)P_[3 * i + 1], (float)P_[3 * i + 2]) : -1;
   const int before = __shfl_up_sync(0xffffffffu, c, 1);
-  const unsigned j = __ballot_sync(0xffffffffu, on && lane > 0 && c != before);
   const unsigned same = __match_any_sync(0xffffffffu, c);
   if (on) {
     o.cell[i] = c;
     if (lane == __ffs(same) - 1) atomicAdd(&o.buckets[c], (unsigned)__popc(same));
   }
-  if (lane == 0 && j) atomicAdd(o.jumps, (unsigned)__popc(j));
-}
-
-static __global__ void k_points_scan(PointOrder o, int64_t n) {
-  grid_dep_wait();
-  grid_dep_launch();
-  if (points_sorted(o, n)) scan_buckets(o.buckets);
-}
-
-static __global__ void k_points_place(PointOrder o, int64_t n) {
-  grid_dep_wait();
-  grid_dep_launch();
-  if (!points_sorted(o, n)) return;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) o.place[i] = (int)atomicAdd(&o.buckets[o.cell[i]], 1u);
+  __threadfence();
+  const int jumps = __syncthreads_count(on && lane > 0 && !cells_touch(c, before));
+  __shared__ bool s_scan;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long add = 1ull << 32 | (unsigned)jumps, sum = atomicAdd(o.tally, add) + add;
+    s_scan = (unsigned)(sum >> 32) == gridDim.x && (int64_t)(unsigned)sum * 4 > n;
+  }
+  __syncthreads();
+  if (!s_scan) return;
+  __threadfence();
+  scan_buckets(o.buckets);
 }
 
 template <class P, typename T>
@@ -2101,7 +2125,9 @@ __global__ void k_points_in(const T* P_, int64_t n, typename P::Vtx* v, PointOrd
   P::set_pos(x, (double)P_[3 * i], (double)P_[3 * i + 1], (double)P_[3 * i + 2]);
   x.tri = -2;
   x.hint = -1;
-  v[points_sorted(o, n) ? o.place[i] : i] = x;
+  int64_t at = i;
+  if (points_sorted(o, n)) o.place[i] = (int)(at = atomicAdd(&o.buckets[o.cell[i]], 1u));
+  v[at] = x;
 }
 
 template <class P>
@@ -2151,21 +2177,21 @@ template <class P>
 int nearest_points(const hd_bvh* B, const void* Pts, int ptype, int64_t n, cudaStream_t s, double* dist,
                    int32_t* idx, double* foot, double* dlo) {
   const bool two_phase = n <= INT32_MAX / 2;  // k_query counts in int
-  const bool sort_list = two_phase && n >= kSortMin, sort_in = two_phase && n >= kPointSortMin;
-  // one allocation: the records, the lists of the two phases, the points' places, and what
-  // starts at zero (run state, jumps, cell counters) at the end
+  const bool sort_in = two_phase && n >= kPointSortMin, sort_list = two_phase && n >= kSortMin && !sort_in;
+  // one allocation: the records, the list of handed-off queries, its reordered copy or the
+  // points' places, and what starts at zero (run state, tally, cell counters) at the end
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t b_rec = up(sizeof(typename P::Vtx) * n), b_list = two_phase ? up(sizeof(int) * n) : 0,
-               b_sorted = sort_list ? b_list : 0, b_place = sort_in ? b_list : 0, b_st = up(sizeof(RunState) + 4),
-               b_buckets = sort_list ? sizeof(unsigned) * kSortBuckets : 0;
+               b_order = sort_list || sort_in ? b_list : 0, b_st = up(sizeof(RunState) + 8),
+               b_buckets = sort_list || sort_in ? sizeof(unsigned) * kSortBuckets : 0;
   char* base = nullptr;
-  HD_TRY(cudaMallocAsync((void**)&base, b_rec + b_list + b_sorted + b_place + b_st + b_buckets, s));
+  HD_TRY(cudaMallocAsync((void**)&base, b_rec + b_list + b_order + b_st + b_buckets, s));
   typename P::Vtx* tmp = (typename P::Vtx*)base;
   int* list = two_phase ? (int*)(base + b_rec) : nullptr;
-  int* sorted = sort_list ? (int*)(base + b_rec + b_list) : nullptr;
-  char* zero = base + b_rec + b_list + b_sorted + b_place;
+  int* order = b_order ? (int*)(base + b_rec + b_list) : nullptr;
+  char* zero = base + b_rec + b_list + b_order;
   RunState* st = (RunState*)zero;
-  unsigned* buckets = sort_list ? (unsigned*)(zero + b_st) : nullptr;
+  unsigned* buckets = b_buckets ? (unsigned*)(zero + b_st) : nullptr;
   cudaError_t e = cudaMemsetAsync(zero, 0, b_st + (sort_in ? b_buckets : 0), s);
   if (e != cudaSuccess) {
     cudaFreeAsync(base, s);
@@ -2173,16 +2199,15 @@ int nearest_points(const hd_bvh* B, const void* Pts, int ptype, int64_t n, cudaS
   }
   PointOrder o;
   if (sort_in) {  // the cells stay in the list's room until the queries start
-    o.place = (int*)(base + b_rec + b_list + b_sorted);
+    o.place = order;
     o.cell = list;
     o.buckets = buckets;
-    o.jumps = (unsigned*)(zero + sizeof(RunState));
+    o.tally = (unsigned long long*)(zero + b_st - 8);
+    const unsigned g = blocks_for(n, kPointCellBlock);
     if (ptype == HD_F64)
-      launch_chained(k_points_cell<double>, blocks_for(n, 256), 256, 0, s, bvh_dev(B), (const double*)Pts, n, o);
+      launch_chained(k_points_cell<double>, g, kPointCellBlock, 0, s, bvh_dev(B), (const double*)Pts, n, o);
     else
-      launch_chained(k_points_cell<float>, blocks_for(n, 256), 256, 0, s, bvh_dev(B), (const float*)Pts, n, o);
-    launch_chained(k_points_scan, 1, 1024, 0, s, o, n);
-    launch_chained(k_points_place, blocks_for(n, 256), 256, 0, s, o, n);
+      launch_chained(k_points_cell<float>, g, kPointCellBlock, 0, s, bvh_dev(B), (const float*)Pts, n, o);
   }
   if (ptype == HD_F64)
     launch_chained(k_points_in<P, double>, blocks_for(n, 256), 256, 0, s, (const double*)Pts, n, tmp, o);
@@ -2190,7 +2215,7 @@ int nearest_points(const hd_bvh* B, const void* Pts, int ptype, int64_t n, cudaS
     launch_chained(k_points_in<P, float>, blocks_for(n, 256), 256, 0, s, (const float*)Pts, n, tmp, o);
   {
     TraceScope tr(HD_K_QUERY, s);
-    query_points<P>(bvh_dev(B), tmp, n, st, list, s, sorted, buckets);
+    query_points<P>(bvh_dev(B), tmp, n, st, list, s, sort_list ? order : nullptr, sort_list ? buckets : nullptr);
   }
   launch_chained(k_points_out<P>, blocks_for(n, 256), 256, 0, s, (const typename P::Vtx*)tmp, n, (const int4*)B->tri_vid,
                  dist, idx, foot, dlo, o);
