@@ -140,7 +140,9 @@ constexpr int kMaxWarps = 32;  // warps of a block
 // lane by lane instead.  There such warps hold many pairs, each a pass of the reductions, and
 // the lanes' additions spread over as many states; with fewer pairs they meet in a few and are
 // what the reductions are for.  128 pairs: 46.2 ms with reductions, 62.0 lane by lane; 512
-// pairs: 207.1 and 197.5 ms.
+// pairs: 207.5 and 198.3 ms.  The UpperBound kernels, which have no registers to spare, are
+// instantiated for either form (with both in one kernel the bounds of 128 pairs took 17.7 ms
+// instead of 16.1); the others choose at run time.
 constexpr int kAccDirectPairs = 256;
 
 __device__ inline void acc_reset(PairAcc& a, int pair) {
@@ -195,13 +197,13 @@ __device__ inline unsigned long long group_max(unsigned g, float v) {
 // Adds the lanes' deltas to their pairs.  Every lane of the warp must call it (pair -1:
 // nothing to add); `a` is the warp's accumulator.  l stays non-negative (a certified vertex
 // distance less its slack can be below 0), which the maximum on its bits needs.
-template <class P>
+template <int kDirect = -1, class P>
 __device__ inline void acc_batch(PairAcc& a, const BatchCtx& x, int pair, const PairDelta<P>& d, bool long_pass = false) {
   RunState* sts = x.sts;
   const int lane = threadIdx.x & 31;
   if (d.c.err && pair >= 0) atomicExch(&sts[pair].err, 1);
   unsigned left = __ballot_sync(0xffffffffu, pair >= 0);
-  if (x.npairs >= kAccDirectPairs && warp_pair(pair) == -2) {
+  if ((kDirect < 0 ? x.npairs >= kAccDirectPairs : kDirect > 0) && warp_pair(pair) == -2) {
     if (pair >= 0) {
       PairAcc b;
       acc_reset(b, pair);
@@ -521,7 +523,7 @@ inline size_t batch_rebin_smem(int block) {
   return HD_BATCH_REBIN ? (size_t)(block / 32) * kRebinQueue * sizeof(BatchRebinEntry) : 0;
 }
 
-template <class P, class Make>
+template <class P, int kDirect, class Make>
 __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vtx* pool, int64_t count, int* counter,
                                          typename P::Item* next, int* next_pair, int next_cap, typename P::Item* u4list,
                                          int* u4_pair, BatchRebinEntry* q, Make make) {
@@ -558,7 +560,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
             classify_pair<P>(x.bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
           }
         }
-        acc_batch(acc, x, need ? -1 : p, ty);
+        acc_batch<kDirect>(acc, x, need ? -1 : p, ty);
         const unsigned m = __ballot_sync(0xffffffffu, need);
         if (need) q[qn + __popc(m & lt)] = e;
         qn += __popc(m);
@@ -586,7 +588,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
       }
       qn -= take;
       __syncwarp();  // the entries taken are read before new ones overwrite them
-      acc_batch(acc, x, p, ty);
+      acc_batch<kDirect>(acc, x, p, ty);
     }
   }
   acc_end(acc, x.sts);
@@ -594,7 +596,7 @@ __device__ inline void batch_bound_rebin(const BatchCtx& x, const typename P::Vt
 
 // UpperBound of the round-0 items: every face of every pair (tri == nullptr), or n given
 // index triples with their pairs (the promoted items of the FP64 phase).
-template <class P, bool kPaper = false>
+template <class P, bool kPaper, int kDirect>
 __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::Vtx* pool, const int32_t* tri,
                                                   const int* tri_pair, int n, typename P::Item* next, int* next_pair,
                                                   int next_cap, typename P::Item* u4list, int* u4_pair) {
@@ -604,7 +606,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
   const int count = tri ? n : x.nF;
   if constexpr (kPaper && HD_BATCH_REBIN) {
     extern __shared__ BatchRebinEntry batch_rebin_q[];
-    batch_bound_rebin<P>(x, pool, count, &bs->b_next, next, next_pair, next_cap, u4list, u4_pair,
+    batch_bound_rebin<P, kDirect>(x, pool, count, &bs->b_next, next, next_pair, next_cap, u4list, u4_pair,
                          batch_rebin_q + (threadIdx.x >> 5) * kRebinQueue,
                          [&](int64_t f, typename P::Item& it, float&) -> int {
                            if (tri) {
@@ -662,7 +664,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_faces(BatchCtx x, const typename P::
       it.U = bound_item<P, kPaper>(x.pd[p].B, pool, it, pl.lv, pl.rp, code, ty.c);
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    acc_batch(acc, x, p, ty);
+    acc_batch<kDirect>(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }
@@ -807,7 +809,7 @@ __global__ void k_batch_select(BatchCtx x, const typename P::Item* front, const 
 
 // The four children of every split (Section 4, midpoint subdivision), bounded with their
 // pair's l and clamped to their parent's U.
-template <class P, bool kPaper = false>
+template <class P, bool kPaper, int kDirect>
 __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename P::Vtx* pool, const int4* split_par,
                                                      const int* split_pair, typename P::Item* next, int* next_pair,
                                                      int next_cap, typename P::Item* u4list, int* u4_pair) {
@@ -819,7 +821,7 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
   const int S = min(*(volatile int*)&bs->n_split, bs->K);
   if constexpr (kPaper && HD_BATCH_REBIN) {
     extern __shared__ BatchRebinEntry batch_rebin_q[];
-    batch_bound_rebin<P>(x, pool, 4 * (int64_t)S, &bs->b_next, next, next_pair, next_cap, u4list, u4_pair,
+    batch_bound_rebin<P, kDirect>(x, pool, 4 * (int64_t)S, &bs->b_next, next, next_pair, next_cap, u4list, u4_pair,
                          batch_rebin_q + (threadIdx.x >> 5) * kRebinQueue,
                          [&](int64_t t, typename P::Item& it, float& up) -> int {
                            const int s = (int)(t >> 2), k = (int)(t & 3);
@@ -866,20 +868,22 @@ __global__ void HD_BOUND_REGS k_batch_bound_children(BatchCtx x, const typename 
       if (pl.rp.parent_clamp && Up < it.U) it.U = Up;
       classify_pair<P>(bs, it, p, pl.lv.th, code, next, next_pair, next_cap, u4list, u4_pair, ty);
     }
-    acc_batch(acc, x, p, ty);
+    acc_batch<kDirect>(acc, x, p, ty);
   }
   acc_end(acc, x.sts);
 }
 
 // The UpperBound kernels of policy P: the straight-line paper-order instantiation or the
-// general one.
+// general one, with the sums of a batch of this many pairs.
 template <class P>
-auto batch_faces_kernel(bool paper) {
-  return paper ? k_batch_bound_faces<P, true> : k_batch_bound_faces<P, false>;
+auto batch_faces_kernel(bool paper, int npairs) {
+  if (npairs >= kAccDirectPairs) return paper ? k_batch_bound_faces<P, true, 1> : k_batch_bound_faces<P, false, 1>;
+  return paper ? k_batch_bound_faces<P, true, 0> : k_batch_bound_faces<P, false, 0>;
 }
 template <class P>
-auto batch_children_kernel(bool paper) {
-  return paper ? k_batch_bound_children<P, true> : k_batch_bound_children<P, false>;
+auto batch_children_kernel(bool paper, int npairs) {
+  if (npairs >= kAccDirectPairs) return paper ? k_batch_bound_children<P, true, 1> : k_batch_bound_children<P, false, 1>;
+  return paper ? k_batch_bound_children<P, true, 0> : k_batch_bound_children<P, false, 0>;
 }
 
 // ----------------------------------------------------------------------------- round control
@@ -1160,7 +1164,7 @@ int batch_rounds(const BatchCtx& x, BatchBufs<P>& R, const BatchCtl& c, int n_po
     if (rh != HD_OK) return rh;
   }
   const bool paper = paper_cascade(x.rp);
-  auto k_children = batch_children_kernel<P>(paper);
+  auto k_children = batch_children_kernel<P>(paper, x.npairs);
   const size_t smem_b = batch_rebin_smem(bs_);  // the u3 queues of the paper-order kernels
   const unsigned g_q = batch_grid(k_batch_query<P>, bs_, sms), g_b = batch_grid(k_children, bs_, sms, smem_b);
   const unsigned g_long = batch_grid(k_batch_query_long<P>, 32 * kCoopWarps, sms);
@@ -1266,7 +1270,7 @@ int batch_finish_fp64(const BatchCtx& xm, BatchBufs<P>& RM, int64_t n_pro, const
   }
   {
     TraceScope tr(HD_K_BOUND, s);
-    launch_chained(batch_faces_kernel<PolicyD>(paper_cascade(x.rp)), blocks_for(n_pro, bsz), bsz, batch_rebin_smem(bsz),
+    launch_chained(batch_faces_kernel<PolicyD>(paper_cascade(x.rp), x.npairs), blocks_for(n_pro, bsz), bsz, batch_rebin_smem(bsz),
                    s, x, (const VtxD*)D.pool, (const int32_t*)tris, (const int*)tri_pair, (int)n_pro, D.front[1],
                    D.front_pair[1], (int)D.front_cap, D.left(1), D.left_pair(1));
     launch_chained(k_batch_bound_u4<PolicyD>, (unsigned)sms * 8, pass_block<PolicyD>(bsz), 0, s, x, (const VtxD*)D.pool,
@@ -1426,7 +1430,7 @@ int run_batch(const hd_bvh* const* Bs, const hd_mesh* As, int64_t npairs, double
   }
   {
     TraceScope tr(HD_K_BOUND, s);
-    auto k_faces = batch_faces_kernel<P>(paper);
+    auto k_faces = batch_faces_kernel<P>(paper, x.npairs);
     launch_chained(k_faces, std::min(blocks_for(nF, bsz), batch_grid(k_faces, bsz, sms, batch_rebin_smem(bsz))), bsz,
                    batch_rebin_smem(bsz), s, x,
                    (const typename P::Vtx*)R.pool, (const int32_t*)nullptr, (const int*)nullptr, 0, R.front[1],
