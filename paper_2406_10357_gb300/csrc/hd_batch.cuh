@@ -139,11 +139,11 @@ constexpr int kMaxWarps = 32;  // warps of a block
 // Batches of at least this many pairs: a warp whose items belong to more than one pair adds them
 // lane by lane instead.  There such warps hold many pairs, each a pass of the reductions, and
 // the lanes' additions spread over as many states; with fewer pairs they meet in a few and are
-// what the reductions are for.  128 pairs: 46.2 ms with reductions, 62.0 lane by lane; 512
-// pairs: 207.5 and 198.3 ms.  The UpperBound kernels, which have no registers to spare, are
+// what the reductions are for.  With reductions / lane by lane, ms: 128
+// pairs 46.2 / 62.0, 260 95.2 / 100.5, 384 146.1 / 146.5, 448 177.1 / 173.1, 512 207.5 / 198.3.  The UpperBound kernels, which have no registers to spare, are
 // instantiated for either form (with both in one kernel the bounds of 128 pairs took 17.7 ms
 // instead of 16.1); the others choose at run time.
-constexpr int kAccDirectPairs = 256;
+constexpr int kAccDirectPairs = 384;
 
 __device__ inline void acc_reset(PairAcc& a, int pair) {
   a.l = a.uret = a.umax = 0ull;
