@@ -133,8 +133,16 @@ struct PairAcc {
   unsigned long long l, uret, umax;  // bits of non-negative doubles
   unsigned evals, leaf, boxes, escalations, nodes, nq, retired, kept;
   unsigned discards[6];
-  int pair;  // -1: empty
+  int pair;  // -1: empty; with kAccFull: to be added before the next batch
 };
+// A traversal's work is not bounded by its items, so a warp whose 32-bit counts have come half
+// way adds them to the state's 64-bit ones (with 64-bit counts in shared memory 128 pairs took
+// 47.2 ms, 46.1 so).  One batch adds less than the other half.
+constexpr int kAccFull = 1 << 30;
+#ifndef HD_ACC_HALF
+#define HD_ACC_HALF (1u << 31)
+#endif
+constexpr unsigned kAccHalf = HD_ACC_HALF;
 constexpr int kMaxWarps = 32;  // warps of a block
 // Batches of at least this many pairs: a warp whose items belong to more than one pair adds them
 // lane by lane instead.  There such warps hold many pairs, each a pass of the reductions, and
@@ -155,13 +163,13 @@ __device__ inline void acc_reset(PairAcc& a, int pair) {
 // Adds `a` to the state of its pair (one lane).
 __device__ inline void acc_apply(RunState* sts, const PairAcc& a, bool long_pass) {
   if (a.pair < 0) return;
-  RunState* st = sts + a.pair;
-  auto add = [](unsigned long long* p, unsigned v) {
-    if (v) atomicAdd(p, (unsigned long long)v);
+  RunState* st = sts + (a.pair & ~kAccFull);
+  auto add = [](unsigned long long* p, unsigned long long v) {
+    if (v) atomicAdd(p, v);
   };
   if (a.l) atomicMax(&st->l_bits, a.l);
   add(&st->queries, a.nq);
-  add(&st->evals, a.evals + a.leaf);
+  add(&st->evals, (unsigned long long)a.evals + a.leaf);
   add(&st->leaf_tests, a.leaf);
   add(&st->box_tests, a.boxes);
   add(&st->escalations, a.escalations);
@@ -240,12 +248,16 @@ __device__ inline void acc_batch(PairAcc& a, const BatchCtx& x, int pair, const 
       const bool first = lane == __ffs(g) - 1;
       auto sum = [g, first](unsigned& to, unsigned v) {
         const unsigned s = __reduce_add_sync(g, v);
-        if (first) to += s;
+        return first ? (to += s) : 0u;
       };
       sum(a.evals, d.c.evals);
-      sum(a.leaf, d.c.leaf);
-      sum(a.boxes, d.c.boxes);
+      const unsigned t = sum(a.leaf, d.c.leaf), b = sum(a.boxes, d.c.boxes);
       sum(a.nodes, d.c.nodes);
+      // (nodes and escalations are fewer than boxes and leaf tests; a bound's evaluations at
+      // most 21 per item)
+      if constexpr (kDirect < 0) {
+        if (max(t, b) >= kAccHalf) a.pair = p | kAccFull;
+      }
       if (__any_sync(g, d.c.escalations != 0)) sum(a.escalations, d.c.escalations);
       if (__any_sync(g, d.nq != 0)) {
         sum(a.nq, (unsigned)d.nq);
