@@ -74,7 +74,7 @@ __device__ inline int warp_batch(int* counter, int take = 32) {
 // The two 320-triangle spheres in FP64: 1190 -> 836 us per pair; 1000 points, MIXED: 80 -> 49 us
 // (2, 4, 8, 16 warps per SM: 57, 54, 49, 49).  FP64 queries of the two-sided scan with 1, 2, 4,
 // 8: 0.93, 0.87, 0.80, 0.76 ms; its bounds 0.79, 0.78, 0.81, 0.97 ms.
-constexpr int kSms = 152;
+constexpr int kSms = 152;  // GB300's, the only part this library is built for
 __device__ inline int spread_lanes(int64_t count, int per_sm) {
   const int64_t warps = min((int64_t)gridDim.x * (blockDim.x >> 5), (int64_t)per_sm * kSms);
   int lanes = 32;
@@ -736,90 +736,6 @@ __device__ inline typename P::UT bound_item(const BvhDev& B, const typename P::V
     return P::upper_bound(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.l, lv.lf, rp, code, c);
 }
 
-// The paper-order cascade with the items that reach u3 gathered into full warps (MIXED).  The
-// exact case, u1 and u2 are cheap and decide many items; u3 costs 4 to 15 point-triangle
-// evaluations.  Run item by item, the lanes whose items were decided early idle while the
-// others evaluate u3.  Here each warp takes batches of 32 items, runs the cheap part on them,
-// and appends the items that still need u3 to its queue in shared memory (64 entries); when 32
-// are waiting, every lane takes one and finishes it, so u3 runs on full warps.  The values and
-// result codes are those of the item-by-item cascade; only the order of the classification
-// changes.  `make(t, it, up)` gives item t (false: no item) and the bound it is clamped to
-// (its parent's U, or +inf).
-// On for the batched run's kernels (HD_BATCH_REBIN), off for a single run's (HD_REBIN): on the
-// 1024-pair batched workload, where 72% of the child items reach u3, it took the UpperBound
-// kernels from 168 to 155 ms per call; on the torus pair, where most items are decided by the
-// exact case, from 0.091 to 0.098 ms (the queue's traffic costs more than the idle lanes).
-#ifndef HD_REBIN
-#define HD_REBIN 0
-#endif
-#ifndef HD_BATCH_REBIN
-#define HD_BATCH_REBIN 1
-#endif
-struct RebinEntry {
-  int v[3];
-  float u12;  // min(u1, u2)
-  float up;   // clamp
-};
-constexpr int kRebinQueue = 64;  // entries per warp
-inline size_t rebin_smem(int block) { return HD_REBIN ? (size_t)(block / 32) * kRebinQueue * sizeof(RebinEntry) : 0; }
-
-template <class P, class Make>
-__device__ inline void bound_rebin(const BvhDev& B, const typename P::Vtx* pool, int64_t count, int* counter,
-                                   const Level<P>& lv, const RunParams& rp, RunState* st, typename P::Item* next,
-                                   int next_cap, typename P::Item* u4list, RebinEntry* q, Counters& c, Tally<P>& ty,
-                                   Make make) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  int qn = 0;  // entries waiting in this warp's queue (uniform over the warp)
-  bool more = true;
-  while (more || qn > 0) {
-    if (more && qn < 32) {
-      const int64_t base = warp_batch(counter);
-      if (base >= count) {
-        more = false;
-      } else {
-        const int64_t t = base + lane;
-        bool need = false;
-        RebinEntry e;
-        typename P::Item it;
-        float up = INFINITY;
-        if (t < count && make(t, it, up)) {
-          typename P::UT U;
-          float u12;
-          int code;
-          if (P::paper_cheap(B, pool[it.v[0]], pool[it.v[1]], pool[it.v[2]], lv.lf, rp, &U, &code, &u12)) {
-            need = true;
-            e = RebinEntry{{it.v[0], it.v[1], it.v[2]}, u12, up};
-          } else {
-            it.U = up < U ? up : U;
-            classify<P>(st, it, lv.th, code, next, next_cap, u4list, ty);
-          }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, need);
-        if (need) q[qn + __popc(m & lt)] = e;
-        qn += __popc(m);
-        __syncwarp();
-      }
-    }
-    if (qn >= 32 || (!more && qn > 0)) {
-      const int take = min(qn, 32);
-      if (lane < take) {
-        const RebinEntry e = q[qn - take + lane];
-        typename P::Item it;
-        it.v[0] = e.v[0];
-        it.v[1] = e.v[1];
-        it.v[2] = e.v[2];
-        int code;
-        const typename P::UT U = P::paper_u3(B, pool[e.v[0]], pool[e.v[1]], pool[e.v[2]], lv.lf, rp, e.u12, e.up, code, c);
-        it.U = e.up < U ? e.up : U;
-        classify<P>(st, it, lv.th, code, next, next_cap, u4list, ty);
-      }
-      qn -= take;
-      __syncwarp();  // the entries taken are read before new ones overwrite them
-    }
-  }
-}
-
 // Round 0: UpperBound for every face of A.
 template <class P, bool kPaper = false>
 __global__ void HD_BOUND_REGS k_bound_faces(BvhDev B, const typename P::Vtx* pool, const int32_t* FA, int64_t nFA, RunState* st,
@@ -832,21 +748,6 @@ __global__ void HD_BOUND_REGS k_bound_faces(BvhDev B, const typename P::Vtx* poo
   const Thresholds<P>& th = lv.th;
   Counters c;
   Tally<P> ty;
-  if constexpr (kPaper && HD_REBIN) {
-    extern __shared__ RebinEntry rebin_q[];
-    bound_rebin<P>(B, pool, nFA, &st->b_next, lv, rp, st, next, next_cap, u4list, rebin_q + (threadIdx.x >> 5) * kRebinQueue,
-                   c, ty, [&](int64_t f, typename P::Item& it, float&) {
-                     it.v[0] = FA[3 * f];
-                     it.v[1] = FA[3 * f + 1];
-                     it.v[2] = FA[3 * f + 2];
-                     // A is validated concurrently: skip bad rows
-                     return it.v[0] >= 0 && it.v[1] >= 0 && it.v[2] >= 0 && it.v[0] < n_pool_valid &&
-                            it.v[1] < n_pool_valid && it.v[2] < n_pool_valid;
-                   });
-    flush_counters(st, c);
-    flush_tally(st, ty);
-    return;
-  }
   const int lanes = rp.keep_order ? 32 : spread_lanes(nFA, P::kSpreadBounds);
   for (;;) {
     const int64_t base = warp_batch(&st->b_next, lanes);
@@ -1067,26 +968,6 @@ __device__ inline void bound_children_body(BvhDev B, const typename P::Vtx* pool
   const Thresholds<P>& th = lv.th;
   Counters c;
   Tally<P> ty;
-  if constexpr (kPaper && HD_REBIN) {
-    extern __shared__ RebinEntry rebin_q[];
-    bound_rebin<P>(B, pool, 4 * (int64_t)S, &st->b_next, lv, rp, st, next, next_cap, u4list,
-                   rebin_q + (threadIdx.x >> 5) * kRebinQueue, c, ty,
-                   [&](int64_t t, typename P::Item& it, float& up) {
-                     const int s = (int)(t >> 2), k = (int)(t & 3);
-                     const int4 par = split_par[s];
-                     const int4 mid = share ? split_mid[s] : make_int4(mbase + 3 * s, mbase + 3 * s + 1, mbase + 3 * s + 2, 0);
-                     if (k == 0) { it.v[0] = par.x; it.v[1] = mid.x; it.v[2] = mid.z; }
-                     else if (k == 1) { it.v[0] = mid.x; it.v[1] = par.y; it.v[2] = mid.y; }
-                     else if (k == 2) { it.v[0] = mid.z; it.v[1] = mid.y; it.v[2] = par.z; }
-                     else { it.v[0] = mid.x; it.v[1] = mid.y; it.v[2] = mid.z; }
-                     // the child lies inside its parent: h(child, B) <= U(parent)
-                     if (rp.parent_clamp) up = __int_as_float(par.w);
-                     return true;
-                   });
-    flush_counters(st, c);
-    flush_tally(st, ty);
-    return;
-  }
   const int lanes = rp.keep_order ? 32 : spread_lanes(4 * (int64_t)S, P::kSpreadBounds);
   for (;;) {
     const int64_t base = warp_batch(&st->b_next, lanes);
@@ -1276,6 +1157,7 @@ constexpr int kTailCluster = HD_TAIL_CLUSTER;  // blocks (8: the largest portabl
 #endif
 constexpr int kTailLong = HD_TAIL_LONG;  // most long queries a round may hand off and stay in the small-round kernel
 constexpr size_t kTailSmem = (sizeof(unsigned) + sizeof(float)) * kTailWarps * kCoopStack;
+static_assert(kTailSmem <= 48 * 1024, "more has to be asked for");
 
 // Every thread of the cluster; global writes before it are seen by every block after it.
 __device__ inline void tail_sync() {
@@ -1621,21 +1503,6 @@ inline int host_res(HostRes*& out) {
 #define HD_AHEAD_FROM 2  // rounds read before the host keeps one round queued ahead
 #endif
 
-// k_tail_rounds takes more than the default 48 KB of dynamic shared memory: allowed once per
-// device.
-template <class P>
-cudaError_t tail_smem_attr() {
-  static std::atomic<unsigned long long> done{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_tail_rounds<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
-  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
-  return e;
-}
-
 // Frontier rounds of policy P over the items that the bound kernel before it left in
 // R.front[R.cur] (their count in st->n_next), until the frontier is empty, the capacity or
 // round limit is reached, or an error is flagged.  Each round starts with k_round_ctl, which
@@ -1669,9 +1536,8 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
   static std::atomic<unsigned> grid_b_cache[2][33];
   const bool paper = paper_cascade(rp);
   const auto k_children = bound_children_kernel<P>(paper);
-  const size_t smem_b = rebin_smem(bs);  // the u3 queues of the paper-order kernels
   const unsigned grid_q = query_grid<P>(bs),
-                 grid_b = persistent_grid_bs(k_children, bs, grid_b_cache[paper ? 1 : 0], smem_b);
+                 grid_b = persistent_grid_bs(k_children, bs, grid_b_cache[paper ? 1 : 0]);
   const bool cuts = cut_enabled(o);
   int64_t front_bound = first_front_bound;  // the first round is queued without a wait
   int last_long = -1;  // long queries of the last round read (-1: none read yet)
@@ -1715,7 +1581,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     }
     {
       TraceScope tr(HD_K_BOUND, s);
-      launch_chained(k_children, g_b, bs, smem_b, s, B, R.pool, R.split_par, R.split_mid, st, rp, R.front[cur ^ 1],
+      launch_chained(k_children, g_b, bs, 0, s, B, R.pool, R.split_par, R.split_mid, st, rp, R.front[cur ^ 1],
                      (int)R.front_cap, R.left(cur ^ 1));
       launch_chained(k_bound_u4<P>, g_u4, pass_block<P>(bs), 0, s, B, R.pool, (const typename P::Item*)R.left(cur ^ 1),
                      (int)R.front_cap, st, rp, R.front[cur ^ 1], (int)R.front_cap);
@@ -1729,7 +1595,6 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
   const TailBufs<P> tb = {{R.front[0], R.front[1]}, R.split_par, R.split_mid, R.tab, R.pool, R.promo, (int)R.promo_cap,
                           (int)R.front_cap, R.u4list, R.longq};
   auto issue_tail = [&](int slot) -> int {
-    HD_TRY(tail_smem_attr<P>());
     {
       TraceScope tr(HD_K_SMALL, s);
       launch_chained(k_tail_rounds<P>, kTailCluster, kTailThreads, kTailSmem, s, B, tb, st, rp, c, init ? 1 : 0, n_pool0, cur);
@@ -1880,7 +1745,7 @@ int finish_in_fp64(const RunIO& io, Rounds<P>& RM, int64_t n_pro, RunState* st, 
   {
     TraceScope tr(HD_K_BOUND, s);
     const auto k_faces = bound_faces_kernel<PolicyD>(paper_cascade(rp));
-    launch_chained(k_faces, spread_grid(n_pro, o.block_size, 65535u, PolicyD::kSpreadBounds), o.block_size, rebin_smem(o.block_size), s, B, D.pool, tris,
+    launch_chained(k_faces, spread_grid(n_pro, o.block_size, 65535u, PolicyD::kSpreadBounds), o.block_size, 0, s, B, D.pool, tris,
                    n_pro, st, rp, D.front[1], (int)D.front_cap, D.left(1), 3 * n_pro);
     launch_chained(k_bound_u4<PolicyD>, spread_grid(n_pro, pass_block<PolicyD>(o.block_size), 65535u, PolicyD::kSpreadBounds),
                    pass_block<PolicyD>(o.block_size), 0, s, B, D.pool, (const ItemD*)D.left(1), (int)D.front_cap, st, rp,
@@ -1974,10 +1839,8 @@ int run_bnb(const RunIO& io) {
   {
     TraceScope tr(HD_K_BOUND, s);
     const auto k_faces = bound_faces_kernel<P>(paper_cascade(rp));
-    launch_chained(k_faces, spread_grid(io.nFA, bs, persistent_grid(k_faces, bs, sms, rebin_smem(bs)), P::kSpreadBounds), bs,
-                   rebin_smem(bs), s, 
-        B, R.pool, io.FA, io.nFA, st, rp, R.front[1],
-                                                           (int)R.front_cap, R.left(1), io.nVA);
+    launch_chained(k_faces, spread_grid(io.nFA, bs, persistent_grid(k_faces, bs, sms), P::kSpreadBounds), bs, 0, s, B,
+                   R.pool, io.FA, io.nFA, st, rp, R.front[1], (int)R.front_cap, R.left(1), io.nVA);
     launch_chained(k_bound_u4<P>, max_grid, pass_block<P>(bs), 0, s, B, R.pool, (const typename P::Item*)R.left(1),
                    (int)R.front_cap, st, rp, R.front[1], (int)R.front_cap);
   }
