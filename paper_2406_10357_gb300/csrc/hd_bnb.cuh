@@ -1540,7 +1540,8 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
                  grid_b = persistent_grid_bs(k_children, bs, grid_b_cache[paper ? 1 : 0]);
   const bool cuts = cut_enabled(o);
   int64_t front_bound = first_front_bound;  // the first round is queued without a wait
-  int last_long = -1;  // long queries of the last round read (-1: none read yet)
+  int last_long = -1;  // long queries of the last round read (-1: none read yet) ...
+  int64_t last_splits = 1;  // ... and the sub-triangles it split
   int cur = R.cur;
   bool init = true;
   // the run state and parameters after the work queued so far, into ring slot `slot`
@@ -1572,11 +1573,14 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
     {
       TraceScope tr(HD_K_LONG, s);
       // The reordering where this round may hand off a list worth it: not where the last round
-      // read handed off few, of a frontier at least a quarter of this one's bound.
-      // (Left out, the list keeps its order: the reordered copy is not this round's.)
+      // read, scaled by how many more sub-triangles this one may split, handed off less than
+      // half of that.  (Left out, the list keeps its order: the reordered copy is not this
+      // round's.)
       LongList ll = R.longq;
-      if (last_long < 0 || 8 * (int64_t)last_long >= kSortMin) sort_long<P>(B, R.pool, ll, st, true, sms, s, rp.dyn);
-      else ll.sorted = nullptr;
+      if (last_long < 0 || 2 * (double)last_long * (double)k >= (double)kSortMin * (double)last_splits)
+        sort_long<P>(B, R.pool, ll, st, true, sms, s, rp.dyn);
+      else
+        ll.sorted = nullptr;
       launch_query_long<P>(cuts, B, R.pool, ll, st, rp.slack, rp.dyn, true, s);
     }
     {
@@ -1625,6 +1629,7 @@ int loop_rounds(const RunIO& io, Rounds<P>& R, RunState* st, HostRes& hr, const 
       tail_at = -1;
     }
     last_long = h.n_long;
+    last_splits = std::max<int64_t>(1, std::min<int64_t>(h.n_split, h.K));
     ++seen;
     // the next round's frontier is h.n_next; one more round ahead may have up to 4x as many
     front_bound = issued == seen ? (int64_t)h.n_next : std::min<int64_t>(4 * (int64_t)h.n_next, R.front_cap);
