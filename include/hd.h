@@ -129,7 +129,10 @@ typedef struct {
   int64_t rounds;            /* frontier rounds after round 0                              */
   int64_t splits;            /* sub-triangles split 1->4 (Section 4's B&B iterations)      */
   int64_t queries;           /* nearest-triangle queries (vertices of A and midpoints)     */
-  int64_t pointtri_evals;    /* point-triangle distance evaluations (leaf tests + u3)      */
+  int64_t pointtri_evals;    /* point-triangle distance evaluations (leaf tests + u3).  In FP64 one
+                                that an FP32 bound settles counts like one in double, and a
+                                sub-triangle whose u3 both the FP32 filter and the FP64 pass
+                                evaluate counts in each                                     */
   int64_t leaf_tests;        /* ... of which in the BVH traversal (leaf triangles tested)  */
   int64_t box_tests;         /* BVH child-box distance evaluations (one per non-empty child
                                 of each node visited, so up to 4 per node)                 */

@@ -73,7 +73,9 @@ __device__ inline int warp_batch(int* counter, int take = 32) {
 // that way.  The FP64 pipe takes as long for one lane as for 32, so FP64 bounds want few.
 // The two 320-triangle spheres in FP64: 1190 -> 836 us per pair; 1000 points, MIXED: 80 -> 49 us
 // (2, 4, 8, 16 warps per SM: 57, 54, 49, 49).  FP64 queries of the two-sided scan with 1, 2, 4,
-// 8: 0.93, 0.87, 0.80, 0.76 ms; its bounds 0.79, 0.78, 0.81, 0.97 ms.
+// 8: 0.93, 0.87, 0.80, 0.76 ms; its bounds 0.79, 0.78, 0.81, 0.97 ms.  For FP64 bounds 2, 3 and 4
+// lie within 2% of each other on 19 calls (20,000 slivers 8.62, 8.72, 8.88 ms, spheres of 6,400
+// faces 1.09, 1.08, 1.11 ms, the two-sided scan 1.96, 1.97, 1.98 ms).
 constexpr int kSms = 152;  // GB300's, the only part this library is built for
 __device__ inline int spread_lanes(int64_t count, int per_sm) {
   const int64_t warps = min((int64_t)gridDim.x * (blockDim.x >> 5), (int64_t)per_sm * kSms);
@@ -112,8 +114,9 @@ __device__ inline void flush_counters(RunState* st, const Counters& c, bool long
 // edge length of A's faces (for cut_radius; as the bits of a non-negative double, one
 // atomic per block that raises it), with `ev` the longest edge at each vertex.  One face per
 // thread, so that its three vertices are read once (per corner they were read three times:
-// the set-up of a run on 2M faces 73 -> 56 us, on 200,000 faces 27 -> 17 us).  Launched with 256 threads per block on a grid-stride loop (a
-// bounded grid, so that few blocks contend for the edge maximum).
+// the set-up of a run on 2M faces 73 -> 56 us, on 200,000 faces 27 -> 17 us).  Launched with 256
+// threads per block on a grid-stride loop (a bounded grid, so that few blocks contend for the
+// edge maximum).
 template <typename T>
 __global__ void k_mark_ref(const int32_t* FA, int64_t nFA, int64_t nVA, uint8_t* ref, int* bad, const T* VA,
                            unsigned long long* e2max_bits, unsigned* ev) {
@@ -341,8 +344,8 @@ __device__ inline unsigned long_bucket(const BvhDev& B, float px, float py, floa
 
 // Nearest-triangle queries for pool vertices [beg, beg + count); count = min(*count_ptr *
 // mult, cap) when count_ptr is given (device-side counts), else `cap`.  Warps take batches of
-// 32 consecutive vertices (fewer of a short list: spread_lanes), one per lane, each lane traversing on its own (the while-while
-// traversal).  With a list, a lane whose traversal tests more than kLongBudget triangles
+// 32 consecutive vertices (fewer of a short list: spread_lanes), one per lane, each lane
+// traversing on its own (the while-while traversal).  With a list, a lane whose traversal tests more than kLongBudget triangles
 // stops and hands its query to k_query_long, which runs next and counts it.  Registers are
 // capped at 128 (a few spilled to L1), for 8 resident blocks of 64 threads per SM.
 #ifndef HD_QUERY_SEGMENTS
@@ -1143,9 +1146,11 @@ static __global__ void k_round_ctl(RunState* st, RoundCtl c, int init, int n_poo
 // path then takes over, so any frontier is correct.  The phases take their work from the same
 // counters whatever the number of blocks; one block of 256 threads ran these rounds before
 // (last rounds of the 320-triangle spheres in FP64 0.108 -> 0.093 ms, of the two-sided scan
-// 0.175 -> 0.146 ms).  A MIXED pair of 320 triangles took 421, 426, 377, 383 us with a
-// frontier of at most 64, 256, 512, 1024 items, larger pairs the same with any; an FP64 one
-// 691, 707, 901, 905 us: eight SMs' FP64 pipes are too few for more than the smallest rounds.
+// 0.175 -> 0.146 ms).  MIXED pairs of 320 triangles took 419, 420, 374, 376 us with a
+// frontier of at most 64, 256, 512, 1024 items (a torus; spheres 491, 475, 420, 420), 18 larger
+// ones (576 to 200,000 triangles) the same within 2% with 64 to 512 and within 5% either way
+// with 1024; an FP64 pair of 320 took 691, 707, 901, 905 us: eight SMs' FP64 pipes are too few for
+// more than the smallest rounds.
 constexpr int kTailThreads = 256;
 constexpr int kTailWarps = kTailThreads / 32;
 #ifndef HD_TAIL_CLUSTER

@@ -57,8 +57,10 @@ constexpr int kCoopMinBlocks = HD_COOP_MIN_BLOCKS;
 constexpr int kCoopMinBlocksCut = HD_COOP_MIN_BLOCKS_CUT;
 // The FP64 policy's cooperative traversal keeps doubles in flight (its query point, the best
 // squared distance and closest point, the triangle being tested): at 40 registers it spills
-// heavily, so it asks for fewer blocks per SM (40,001 points in a volume with 4, 5, 6, 7, 8
-// blocks: 1.20, 1.23, 1.23, 1.29, 1.27 ms), and its lanes keep their queries longer.
+// heavily, so it asks for fewer blocks per SM, with cuts and without, and its lanes keep their
+// queries longer.  With 3, 4, 6, 8 blocks 40,001 points in a volume took 0.90, 0.87, 0.88, 0.90
+// ms, 300,000 4.65, 4.41, 4.44, 4.45 ms, 20,000 slivers (cut queries) 9.05, 8.72, 9.16, 9.28 ms;
+// pairs and batches whose queries are short differ by under 2%.
 #ifndef HD_COOP_MIN_BLOCKS_D
 #define HD_COOP_MIN_BLOCKS_D 4
 #endif

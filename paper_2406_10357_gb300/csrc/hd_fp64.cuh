@@ -1,5 +1,7 @@
-// FP64 policy: every distance and bound in IEEE double with round-to-nearest, the
-// arithmetic of the paper's implementation (Section 4).
+// FP64 policy: results in IEEE double with round-to-nearest, the arithmetic of the paper's
+// implementation (Section 4).  Comparisons that certified FP32 intervals settle (box distances,
+// leaf triangles, bounds that discard) are settled by them, so that FP64, at 1/64 of the FP32
+// rate, runs where they leave a decision open and for every value that is returned.
 #pragma once
 
 #include "hd_cert.cuh"
