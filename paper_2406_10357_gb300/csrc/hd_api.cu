@@ -151,7 +151,9 @@ int upper_bounds_mixed(const hd_bvh* B, const double* T, const double* Td, const
 // Launched with whole warps: lanes past the last triangle take part in the votes of ub_u3.
 // The distances given need not be those to the triangles given, so u3 has three FP64
 // point-triangle tests of its own to start from; items and orders that do not reach u3 run none
-// (480,000 items, u1 alone: 158 us, 508 with the tests run for every item).
+// (480,000 items, u1 alone: 112 us, 508 with the tests run for every item).  Orders without u3
+// have an instantiation without it: u4 alone 393 us, 467 in the kernel that holds both.
+template <bool kU3>
 __global__ void k_upper_bounds(BvhDev B, const int* inv, const double* T, const double* Td, const int32_t* TI,
                                const double* Tq, int64_t n, double l, RunParams rp, double* U, int32_t* code) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -175,7 +177,7 @@ __global__ void k_upper_bounds(BvhDev B, const int* inv, const double* T, const 
   };
   unsigned ev = 0;
   int c;
-  const double u = upper_bound_d(B, t, own, l, rp.order, rp.n_bounds, true, on, c, ev);
+  const double u = upper_bound_d<kU3>(B, t, own, l, rp.order, rp.n_bounds, true, on, c, ev);
   if (i >= n) return;
   U[i] = on ? u : NAN;
   code[i] = on ? c : -1;
@@ -516,7 +518,9 @@ int hd_upper_bounds(const hd_bvh* B, const double* T, const double* Td, const in
   rp.n_bounds = o.n_bounds;
   cudaStream_t s = (cudaStream_t)stream;
   if (o.precision == HD_MIXED) return upper_bounds_mixed(B, T, Td, TI, Tq, n, l, rp, s, U, code);
-  k_upper_bounds<<<blocks_for(n, 128), 128, 0, s>>>(bvh_dev(B), B->inv, T, Td, TI, Tq, n, l, rp, U, code);
+  const bool u3 = memchr(o.order, 3, o.n_bounds) != nullptr;
+  (u3 ? k_upper_bounds<true> : k_upper_bounds<false>)<<<blocks_for(n, 128), 128, 0, s>>>(bvh_dev(B), B->inv, T, Td, TI, Tq, n,
+                                                                                         l, rp, U, code);
   HD_TRY_LAUNCH();
   return HD_OK;
 }

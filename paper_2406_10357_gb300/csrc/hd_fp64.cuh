@@ -662,8 +662,8 @@ __device__ inline double ub_u4(const VI t[3], double cap) {
 // UpperBound(T, l) of Section 4; own(i) = d(v_i, S_i), asked for only where u3 is reached.  Must
 // be called by all 32 lanes of the warp (ub_u3 votes); lanes with on == false return +inf.
 // With `full`, every bound is evaluated in full (a discarded T then returns the deciding bound's
-// own value).
-template <class Own>
+// own value).  kU3: the order may hold u3.
+template <bool kU3 = true, class Own>
 __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const Own& own, double l, const uint8_t* order,
                                        int nb, bool full, bool on, int& code, unsigned& evals) {
   double U = INFINITY;
@@ -678,13 +678,15 @@ __device__ inline double upper_bound_d(const BvhDev& B, const VI t[3], const Own
     double u = INFINITY;
     const double cap = full ? INFINITY : U;
     if (order[k] == 3) {
-      double d[3] = {0.0, 0.0, 0.0};
-      if (on) {
+      if constexpr (kU3) {
+        double d[3] = {0.0, 0.0, 0.0};
+        if (on) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) d[i] = own(i);
+          for (int i = 0; i < 3; ++i) d[i] = own(i);
+        }
+        const double u3 = ub_u3(B, t, d, cap, on, evals);
+        if (on) u = u3;
       }
-      const double u3 = ub_u3(B, t, d, cap, on, evals);
-      if (on) u = u3;
     } else if (on) {
       u = order[k] == 1 ? ub_u1(t, E) : order[k] == 2 ? ub_u2(t, E, cap) : ub_u4(t, cap);
     }
