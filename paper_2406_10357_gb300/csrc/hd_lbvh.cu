@@ -696,7 +696,9 @@ __global__ void k_emit(int64_t n, int L, const int* left, const int* right, cons
   const int lane = threadIdx.x & 31;
   const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, node0 = node - lane;
   float4* row = stage[threadIdx.x >> 5] + 9 * lane;
-  if (node < n - 1 && last[node] - first[node] + 1 > L) {
+  const bool inner = node < n - 1 && last[node] - first[node] + 1 > L;  // (a node below the leaves is not written)
+  const unsigned rows = __ballot_sync(0xffffffffu, inner);
+  if (inner) {
     float lo0[3], hi0[3], lo1[3], hi1[3];
     int cl = left[node], cr = right[node];
     load_box(cl >= 0 ? ibox + 2 * cl : leafbox + 2 * (int64_t)(~cl), lo0, hi0);
@@ -717,16 +719,13 @@ __global__ void k_emit(int64_t n, int L, const int* left, const int* right, cons
     const float4* src = reinterpret_cast<const float4*>(&nd);
 #pragma unroll
     for (int k = 0; k < 8; ++k) row[k] = src[k];
-  } else {  // a node below the leaves: never visited
-#pragma unroll
-    for (int k = 0; k < 8; ++k) row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __syncwarp();
   float4* out = reinterpret_cast<float4*>(nodes + node0);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int e = 32 * k + lane;  // 16-byte piece of the warp's nodes
-    if (node0 + (e >> 3) < n - 1) out[e] = stage[threadIdx.x >> 5][9 * (e >> 3) + (e & 7)];
+    if (rows >> (e >> 3) & 1u) out[e] = stage[threadIdx.x >> 5][9 * (e >> 3) + (e & 7)];
   }
 }
 
