@@ -298,22 +298,24 @@ __device__ inline float ubm_u2(const VM t[3], const EdgesM& E) {
 }
 
 // Lower bound of u2 for every g its acute test may choose: g is at least half the longest edge,
-// and the circumradius (rounded down) where T is certainly acute.  0 where an edge leaves the
-// float range.
-__device__ inline float ubm_u2_lo(const VM t[3], const EdgesM& E) {
+// and the circumradius (rounded down) where T is certainly acute, which is asked only where
+// the former stays below `enough`.  0 where an edge leaves the float range.
+__device__ inline float ubm_u2_lo(const VM t[3], const EdgesM& E, float enough) {
   float lo[3];  // norm_ru is within 2^-18 above the length, or 1e-15 of it (sqrt_up)
 #pragma unroll
   for (int i = 0; i < 3; ++i) lo[i] = fmaxf(__fsub_rd(__fmul_rd(E.hi[i], 1.f - 0x1p-18f), 2e-15f), 0.f);
   const float hk = fmaxf(E.hi[0], fmaxf(E.hi[1], E.hi[2]));
   if (!(hk < INFINITY)) return 0.f;
+  const float d = __fmul_rd(fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi)), 1.f - 0x1p-20f);
   float g = 0.5f * fmaxf(lo[0], fmaxf(lo[1], lo[2]));
-  if (__fmaf_rd(lo[0], lo[0], __fmaf_rd(lo[1], lo[1], __fmul_rd(lo[2], lo[2]))) > __fmul_ru(__fmul_ru(2.f, hk), hk)) {
+  if (__fadd_rd(g, d) < enough &&
+      __fmaf_rd(lo[0], lo[0], __fmaf_rd(lo[1], lo[1], __fmul_rd(lo[2], lo[2]))) > __fmul_ru(__fmul_ru(2.f, hk), hk)) {
     const F3 a = E.e[2], b = {-E.e[1].x, -E.e[1].y, -E.e[1].z};
     const F3 cr = {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
     const float c2 = __fadd_ru(norm_ru(cr), __fmul_ru(__fmul_ru(32.f * kU, amax3(a)), amax3(b)));  // 2|T|, rounded up
     g = fmaxf(g, div_dn(__fmul_rd(__fmul_rd(lo[0], lo[1]), lo[2]), __fmul_ru(2.f, c2)));
   }
-  return __fadd_rd(g, __fmul_rd(fmaxf(t[0].dhi, fmaxf(t[1].dhi, t[2].dhi)), 1.f - 0x1p-20f));
+  return __fadd_rd(g, d);
 }
 
 // Lower bound of u4 whichever edge of T is taken for the shortest: H(q_i, q_j) is at least the

@@ -906,20 +906,21 @@ struct PolicyD {
     vertices_m(a, b, c, t);
     const Limits m = limits(B, t, lf, rp);
     const EdgesM E(t);
-    const float u1 = ubm_u1(t, E), u2 = ubm_u2(t, E);
+    const float u1 = ubm_u1(t, E);
     int v = verdict(m, u1, u1);
     *code = 1;
     *U = (UT)u1;
     if (v == 0) {
-      v = verdict(m, u2, ubm_u2_lo(t, E));
+      const float u2 = ubm_u2(t, E);
+      v = verdict(m, u2, u2 < m.u12 ? 0.f : ubm_u2_lo(t, E, m.keep));
       *code = 2;
       *U = (UT)u2;
+      *u12 = fminf(u1, u2);
     }
     if (v < 0) {
       *code = kDeferU4;
       *U = INFINITY;
     }
-    *u12 = fminf(u1, u2);
     return v == 0;
   }
   __device__ static UT paper_u3(const BvhDev& B, const Vtx& a, const Vtx& b, const Vtx& c, float lf, const RunParams& rp,
@@ -959,7 +960,7 @@ struct PolicyD {
         v = verdict(m, u, u);
       } else if (o == 2) {
         u = ubm_u2(t, E);
-        v = verdict(m, u, ubm_u2_lo(t, E));
+        v = verdict(m, u, ubm_u2_lo(t, E, m.keep));
       } else if (o == 3) {
         if (m.u3 > 0.f) u = ubm_u3<true>(B, t, m.u3, cnt.evals);
         v = u < m.u3 ? 1 : -1;
