@@ -549,8 +549,8 @@ __global__ void k_long_hist(BvhDev B, const typename P::Vtx* pool, LongList ll, 
 
 // Exclusive scan of the cell counts: one block of 1024 threads, each warp a run of 1024
 // consecutive counters, all loaded first (coalesced) and scanned in registers, so that only the
-// warps' totals wait at a barrier.  (Row after row across the block, with four barriers
-// each, it took 14 us of the 16 it added to a call of hd_nearest.)
+// warps' totals wait at a barrier.  (Row after row across the block, with four barriers each,
+// k_points_cell took 22 us on 131,072 points in random order, 13 so; 5 where it does not scan.)
 __device__ inline void scan_buckets(unsigned* buckets) {
   constexpr int kPer = kSortBuckets / (4 * 1024);
   static_assert(4 * 1024 * kPer == kSortBuckets, "whole rows");
